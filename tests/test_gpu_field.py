@@ -79,6 +79,30 @@ def test_mul_second_operand_any_256_bit_value(F):
 
 
 @pytest.mark.parametrize("F", FIELDS, ids=lambda f: f.name)
+def test_mul_carry_chains(F):
+    """Operands made of limbs 0, 1, 2^31, 2^32 - 1 and the modulus's own: rows
+    whose reduction multiplier is zero, and carries that run the length of a
+    chain."""
+    import paper_2509_22684_gb300 as zk
+    n, r = 1 << 15, F.r
+    words = splitmix64(41, 0, 16 * n).reshape(n, 2, 8)
+    vals = [0, 1, 1 << 31, 0xFFFFFFFF]
+    A, B = [], []
+    for i in range(n):
+        v = []
+        for s in range(2):
+            limbs = [(vals + [(r >> (32 * k)) & 0xFFFFFFFF])[int(words[i, s, k]) % 5] for k in range(8)]
+            v.append(sum(l << (32 * k) for k, l in enumerate(limbs)))
+        A.append(v[0] % r)
+        B.append(v[1])
+    got = limbs_to_ints(to_host(zk.field_op(F.name, "mul", to_dev(ints_to_limbs(A)),
+                                            to_dev(ints_to_limbs(B)))))
+    want = [F.mont_mul(x, y) for x, y in zip(A, B)]
+    bad = [i for i in range(n) if got[i] != want[i]]
+    assert not bad, f"{len(bad)} mismatches, first at {bad[0]}: {A[bad[0]]:x} {B[bad[0]]:x}"
+
+
+@pytest.mark.parametrize("F", FIELDS, ids=lambda f: f.name)
 def test_pointwise(F):
     import paper_2509_22684_gb300 as zk
     n = 4096
