@@ -78,15 +78,11 @@ typedef struct {
     int use_tuner;         /* 0 or 1: use a tuned schedule when one is known for this GPU
                               (zkntt_tuned.jsonl beside the library, then ZKNTT_TUNE_CACHE);
                               -1: never (planner heuristic only) */
-    int ilp;               /* kernel variant: 1 = one butterfly per thread per stage step (3 blocks
-                              per SM), 2 = two interleaved butterflies (2 blocks), 3 = one
-                              butterfly with registers for 4 blocks, 4 = software-pipelined
-                              stage loop (2 blocks), 5 = as 3 with twice the threads per
-                              tile (for small transforms), 6 = as 3 with two tile
-                              buffers (the next tile's loads overlap this tile's
-                              arithmetic), 7 = as 1 with the stages of pair distance
-                              16, 8 and 4 exchanged by warp shuffles instead of shared
-                              memory; 0 = auto; outside 0..7 -> ZKNTT_EINVAL */
+    int ilp;               /* kernel variant: two stages at a time, four elements a thread, with
+                              registers for 3 (1, 3, 6 and 7) or 2 (2 and 4) blocks of 256
+                              threads per SM; 5 = one butterfly per thread per stage,
+                              registers for 4 blocks (for small transforms);
+                              0 = auto; outside 0..7 -> ZKNTT_EINVAL */
 } zkntt_plan_options;
 
 /*

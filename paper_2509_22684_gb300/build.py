@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 INCLUDE = os.path.join(ROOT, "include")
-# ZKNTT_NVCC_FLAGS adds compile flags (e.g. -DZKNTT_BATCH_PAIR=0) and
+# ZKNTT_NVCC_FLAGS adds compile flags (e.g. -DZKNTT_BATCH_MIN_BLOCKS=3) and
 # ZKNTT_LIB_OUT names another output library, for building variants side by side
 EXTRA = os.environ.get("ZKNTT_NVCC_FLAGS", "").split()
 LIB = os.environ.get("ZKNTT_LIB_OUT") or os.path.join(HERE, "libzkntt.so")

@@ -8,29 +8,41 @@
 
 namespace zkntt {
 
+// -r^-1 mod 2^256, by value
+struct NegInv {
+    uint32_t v[8];
+};
+
 // out[i] = hi[i >> split] * lo[i & (2^split - 1)]: the powers b^i from two
-// small tables (b^(i_hi * 2^split) and b^i_lo)
+// small tables (b^(i_hi * 2^split) and b^i_lo), in Montgomery form or (factors)
+// as factors
 template <class F>
 __global__ void gen_powers_kernel(uint4 *out, uint32_t count, const uint4 *hi, const uint4 *lo,
-                                  uint32_t split) {
+                                  uint32_t split, uint32_t factors, const NegInv ninv) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
         uint32_t a[8], b[8];
         ldg_elem(a, hi + 2 * size_t(i >> split));
         ldg_elem(b, lo + 2 * size_t(i & ((1u << split) - 1u)));
         mul<F>(a, a, b);
-        st_elem(out + 2 * size_t(i), a);
+        if (factors) {
+            Factor f;
+            make_factor<F>(f, a, ninv.v);
+            st_factor(out + 4 * size_t(i), f);
+        } else {
+            st_elem(out + 2 * size_t(i), a);
+        }
     }
 }
 
-// Inter-pass twiddle table, row-major by position d (so a tile of consecutive
+// Inter-pass factor table, row-major by position d (so a tile of consecutive
 // columns lo reads consecutive entries):
 //   out[d * 2^lo_bits + lo] = w^(lo * rev_K(d)) * fl[lo] * fd[d]
 // with w^e = w_hi[e >> split] * w_lo[e & mask] (any scalar factor folded into
-// w_lo by the host).  fl / fd may be null.
+// w_lo by the host), all in Montgomery form.  fl / fd may be null.
 template <class F>
 __global__ void gen_twiddle_kernel(uint4 *out, uint32_t K, uint32_t lo_bits, const uint4 *w_hi,
                                    const uint4 *w_lo, uint32_t split, const uint4 *fl,
-                                   const uint4 *fd) {
+                                   const uint4 *fd, const NegInv ninv) {
     const size_t total = size_t(1) << (lo_bits + K);
     for (size_t idx = size_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
          idx += size_t(gridDim.x) * blockDim.x) {
@@ -49,7 +61,9 @@ __global__ void gen_twiddle_kernel(uint4 *out, uint32_t K, uint32_t lo_bits, con
             ldg_elem(b, fd + 2 * size_t(d));
             mul<F>(a, a, b);
         }
-        st_elem(out + 2 * idx, a);
+        Factor f;
+        make_factor<F>(f, a, ninv.v);
+        st_factor(out + 4 * idx, f);
     }
 }
 

@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, BATCH_MIN_BLOCKS)
                  uint32_t *status) {
     extern __shared__ uint4 smem[];
     __shared__ uint32_t s_item, s_seg, s_stop, s_next;
+    const uint4 *table = nullptr;  // the twiddle table in shared memory
     if (threadIdx.x == 0) s_next = atomicAdd(&ctrl[0], 1u);
     for (;;) {
         if (threadIdx.x == 0) {
@@ -71,17 +72,21 @@ __global__ void __launch_bounds__(BATCH_THREADS, BATCH_MIN_BLOCKS)
         if (s_stop) break;
         const BatchSeg &sg = tab.seg[s_seg];
         const uint32_t tile = s_item - sg.first_item;
-        // one butterfly per thread per stage (as pass variant 5): small tiles
-        // keep twice the threads of the block busy
-        const uint32_t nt = pass_threads_for(sg.a.K, sg.a.log_cols, 5);
-        // with the shared-twiddle pairing (one twiddle load for a thread's two
-        // butterflies of a stage): the fused Groth16 sequences run 1-3% faster
-        // from 2^16 up
-#ifndef ZKNTT_BATCH_PAIR
-#define ZKNTT_BATCH_PAIR 1
-#endif
-        run_tile<F, 1, false, false, ZKNTT_BATCH_PAIR>(sg.a, smem, tile, nt < BATCH_THREADS ? nt : BATCH_THREADS);
-        // run_tile ends with a block barrier: every store of the tile is issued
+        // up to one butterfly per thread per stage (as pass variant 5): small
+        // tiles keep twice the threads of the block busy
+        const uint32_t nt5 = pass_threads_for(sg.a.K, sg.a.log_cols, 5);
+        const uint32_t nt = nt5 < BATCH_THREADS ? nt5 : BATCH_THREADS;
+        // the twiddle table stays while tiles of the same sub-transform follow
+        uint4 *buf = smem + tab.table_units;
+        if (sg.a.w_stage != table) {
+            table = sg.a.w_stage;
+            issue_table_load(sg.a, smem);
+        }
+        issue_tile_load(sg.a, buf, tile, nt);
+        cp_async_wait_all();
+        __syncthreads();
+        run_tile<F, EITHER>(sg.a, smem, buf, tile, nt);
+        __syncthreads();  // every store of the tile is issued, the buffers are free
         if (threadIdx.x == 0) {
             __threadfence();
             const uint32_t retired = atomicAdd(&done[s_seg], 1u) + 1u;

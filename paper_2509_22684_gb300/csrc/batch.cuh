@@ -54,6 +54,7 @@ struct BatchTable {
     uint32_t total_items;
     unsigned long long timeout_ns;
     uint32_t *flags;      // per-transform completion words (may be null)
+    uint32_t table_units; // 16-byte units of shared memory kept for the twiddle table
     uint32_t epoch;       // value written to flags[job] when the job completes
     BatchSeg seg[BATCH_MAX_SEGMENTS];
 };

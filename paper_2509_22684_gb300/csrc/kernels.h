@@ -9,7 +9,7 @@ constexpr int MAX_DIGIT_BITS = 11;  // largest sub-transform a block holds (2^11
 constexpr int MAX_TILE_BITS = 11;   // tiles hold at most 2^11 elements (C x 2^K)
 
 struct FieldKernels {
-    const void *pass[8];  // ntt_pass_kernel<F, V> at index V = 1..7 (digit size is a runtime argument)
+    const void *pass[8];  // the pass kernel of schedule variant 1..7 (digit size is a runtime argument)
     const void *gen_powers;
     const void *gen_twiddle;
     const void *field_op;

@@ -6,9 +6,9 @@
 //   n = 2^L is split into digits k_1 + ... + k_p = L (top digit first).  Pass i
 //   treats the vector as columns: for fixed (hi, lo) the N = 2^K elements at
 //       q = (hi * N + d) * 2^lo_bits + lo,   d = 0..N-1
-//   form one sub-transform.  It is computed by radix-2 decimation-in-frequency
-//   stages (output position d then holds frequency rev(d)) and, for every pass
-//   but the last, multiplied by the inter-pass twiddle w_{n_i}^(lo * rev(d)),
+//   form one sub-transform.  It is computed by decimation-in-frequency stages
+//   (output position d then holds frequency rev(d)) and, for every pass but the
+//   last, multiplied by the inter-pass twiddle w_{n_i}^(lo * rev(d)),
 //   n_i = N * 2^lo_bits.  After the last pass the value at position q is
 //   output bitrev_L(q); the last pass writes it there directly, so the result
 //   is in natural order without a permutation pass.
@@ -16,30 +16,33 @@
 // Inside a thread block: a tile of C columns x N rows (C consecutive lo values,
 // or for the last pass C blocks whose bit-reversed indices are consecutive, so
 // the scattered writes form C*32-byte runs) is copied into shared memory with
-// cp.async.  Stages 0..K-3 run as a loop: each thread takes butterflies
-// (x, y) -> (x + y, (x - y) w) from shared memory and writes them back, so the
-// loop body holds a single inlined Montgomery product and stays resident in
-// the instruction cache.  The difference x - y is formed as x + r - y with no
-// conditional correction: it only feeds the product, as its limb-scanned
-// operand, which may be any value below 2^256 (the product's output is
-// canonical either way).  The last two stages run as one radix-4 step per
-// thread on four neighbouring rows, and the scaled elements are then written
-// to global memory.  All sizes (K, C, the stride) are runtime values: one
-// kernel per field serves every digit size.
+// cp.async.  Two stages at a time then run as radix-4 steps: a thread loads the
+// four rows of a group, takes their four butterflies (x, y) -> (x + y, (x - y) w)
+// in registers and writes them back (a radix-2 step comes first when K is odd).
+// The last step, rows d0..d0+3 with one product by w_4, is followed by the
+// element's output factor and the store to global memory.  Tiles with more than
+// one thread per four elements (small transforms, where warps in flight count)
+// take the stages one by one, one butterfly a thread.
+// The difference x - y is formed as x + r - y with no conditional correction:
+// it only feeds the product, which takes any x below 2r.
+// All sizes (K, C, the stride) are runtime values: one kernel per field serves
+// every digit size.
 //
 // Shared memory holds each element as two 16-byte halves in separate arrays.
-// The slot of (column c, row d) is c*N + (d ^ s) with
-//   s = (7 if bit 3 of d is set) ^ (c << (3 - log2 C))   (low three bits),
-// which keeps the butterfly accesses of every stage (pairs at distance 1, 2, 4
-// and >= 8), the column-major copies and the row-major copies free of bank
-// conflicts.
+// The slot of (column c, row d) is c*N + (d ^ s), with s in the low three bits
+// a linear function of bits 3 and 4 of d and of c (smem_slot), chosen so that
+// the eight lanes of an access fall into different bank groups in every
+// pattern: copies with columns or rows fastest, steps at distance 4 and above,
+// and the last step on rows 4 g + i with columns fastest.
 //
-// Fused per-element factors (one Montgomery product each, only when present):
+// Per-element factors (one product each, only when present), all held as
+// (w, quotient) pairs of 64 bytes for mul_factor:
 //   pre[d]          first pass, on input row d (coset forward shift powers)
-//   pw_b, pw_c      first pass, x <- x * pw_b[q] - pw_c[q] (Groth16 pointwise)
-//   tw[d][lo]       inter-pass twiddles, precomputed, or formed on the fly from
-//                   split-exponent tables (w_hi, w_lo) and optional per-column
-//                   (fl) and per-row (fd) factors
+//   pw_b, pw_c      first pass, x <- x * pw_b[q] - pw_c[q] (Groth16 pointwise;
+//                   these are vectors of elements)
+//   tw[d][lo]       inter-pass twiddles, precomputed, or applied on the fly as
+//                   the factors w_hi, w_lo of the split exponent and optional
+//                   per-column (fl) and per-row (fd) ones
 //   post[d]         last pass, on output position d (inverse / coset scales)
 #pragma once
 #include <cstdint>
@@ -51,8 +54,8 @@ namespace zkntt {
 struct PassArgs {
     const uint4 *in;
     uint4 *out;
-    const uint4 *w_stage; // per stage s: w_N^(j 2^s), j < N/2^(s+1), at offset N - 2^(K-s)
-    const uint4 *tw;      // precomputed inter-pass twiddles [N][2^lo_bits] (row-major by d)
+    const uint4 *w_stage; // the factors w_N^e, e < N/2, as they lie in shared memory (tab_slot)
+    const uint4 *tw;      // precomputed inter-pass factors [N][2^lo_bits] (row-major by d)
     const uint4 *w_hi;    // on-the-fly: w^((e >> split_bits) << split_bits)
     const uint4 *w_lo;    // on-the-fly: w^(e & (2^split_bits - 1)) (times any folded scalar)
     const uint4 *fl;      // on-the-fly: per-column factor (may be null)
@@ -68,7 +71,7 @@ struct PassArgs {
     uint32_t split_bits;  // on-the-fly: width of the low exponent table
     uint32_t log_cols;    // log2 C
     uint32_t last;        // 1: last pass (bit-reversed scatter to natural order)
-    uint32_t otf;         // 1: form inter-pass twiddles on the fly
+    uint32_t otf;         // 1: inter-pass twiddles on the fly
     uint32_t num_tiles;   // tiles in this pass
 };
 
@@ -76,11 +79,18 @@ __device__ __forceinline__ uint32_t brev_bits(uint32_t x, uint32_t bits) {
     return bits == 0 ? 0u : (__brev(x) >> (32 - bits));
 }
 
-// swizzled shared-memory slot of element (column c, row d)
+// Row part of the shared-memory slot (K >= 3): d with its low three bits
+// xor 5 for bit 3 and xor 6 for bit 4.  Linear over xor, so the rows of a group
+// at distances that are powers of two have slots at xor distances.
+__device__ __forceinline__ uint32_t row_slot(uint32_t d) {
+    return d ^ (((d >> 3) & 1u) * 5u) ^ (((d >> 4) & 1u) * 6u);
+}
+
+// shared-memory slot of element (column c, row d)
 __device__ __forceinline__ uint32_t smem_slot(uint32_t c, uint32_t d, uint32_t K, uint32_t lc) {
     if (K < 3) return (c << K) + d;
-    uint32_t s = ((((d >> 3) & 1u) * 7u) ^ (c << (3 - lc))) & 7u;
-    return (c << K) + (d ^ s);
+    const uint32_t s = lc == 3 ? c : lc == 2 ? ((c & 1u) << 1) ^ ((c >> 1) * 5u) : c * 6u;
+    return (c << K) + (row_slot(d) ^ s);
 }
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
@@ -95,16 +105,6 @@ __device__ __forceinline__ void cp_async16_sa(uint32_t s, const void *gmem_src) 
 
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit() {
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-
-// wait until at most N committed groups of this thread's copies are pending
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
 __device__ __forceinline__ void lds_elem(uint32_t x[8], const uint4 *s_lo, const uint4 *s_hi,
@@ -140,39 +140,53 @@ __device__ __forceinline__ size_t tile_dst(const PassArgs &a, uint32_t tile, uin
     return (size_t(brev_bits(d, a.K)) << a.hi_bits) + (size_t(tile) << a.log_cols) + cc;
 }
 
-// Output factor of row position d in column cc: the inter-pass twiddle (times
-// folded factors) or the last pass's post scale.  Returns false when there is
-// no factor.
-template <class F>
-__device__ __forceinline__ bool out_factor(uint32_t f[8], const PassArgs &a, uint32_t tile,
-                                           uint32_t d, uint32_t cc) {
+// The factors of row position d in column cc on the way out: the inter-pass
+// twiddle (precomputed, or up to four factors on the fly) or the last pass's
+// post scale.  A null p[0]: none; a null p[k] ends the list.
+__device__ __forceinline__ void out_factors(const uint4 *p[4], const PassArgs &a, uint32_t tile,
+                                            uint32_t d, uint32_t cc) {
+    p[0] = p[1] = p[2] = p[3] = nullptr;
     if (a.last) {
-        if (!a.post) return false;
-        ldg_elem(f, a.post + 2 * size_t(d));
-        return true;
+        if (a.post) p[0] = a.post + 4 * size_t(d);
+        return;
     }
     const uint32_t lo_tiles_bits = a.lo_bits - a.log_cols;
     const uint32_t lo = ((tile & ((1u << lo_tiles_bits) - 1u)) << a.log_cols) + cc;
     if (!a.otf) {
-        ldg_elem(f, a.tw + 2 * ((size_t(d) << a.lo_bits) + lo));
-        return true;
+        p[0] = a.tw + 4 * ((size_t(d) << a.lo_bits) + lo);
+        return;
     }
     // lo < 2^lo_bits and rev(d) < 2^K, so e < 2^tw_bits = n_i: no reduction
     // (and no overflow: tw_bits <= 32)
     const uint32_t e = lo * brev_bits(d, a.K);
-    uint32_t g[8];
-    ldg_elem(f, a.w_hi + 2 * size_t(e >> a.split_bits));
-    ldg_elem(g, a.w_lo + 2 * size_t(e & ((1u << a.split_bits) - 1u)));
-    mul_call<F>(f, f, g);
-    if (a.fl) {
-        ldg_elem(g, a.fl + 2 * size_t(lo));
-        mul_call<F>(f, f, g);
+    p[0] = a.w_hi + 4 * size_t(e >> a.split_bits);
+    p[1] = a.w_lo + 4 * size_t(e & ((1u << a.split_bits) - 1u));
+    if (a.fl) p[2] = a.fl + 4 * size_t(lo);
+    if (a.fd) (a.fl ? p[3] : p[2]) = a.fd + 4 * size_t(d);
+}
+
+// x times its output factors, to its place in global memory.  One product in
+// the code, in a loop over the factors: unrolled, the kernels outgrow the
+// instruction cache.
+template <class F>
+__device__ __forceinline__ void scale_and_store(uint32_t x[8], const PassArgs &a, uint32_t tile,
+                                                uint32_t d, uint32_t cc) {
+    const uint4 *p[4];
+    out_factors(p, a, tile, d, cc);
+    // an entry of the big table is read once: it takes no place in L1
+    const bool stream = !a.last && !a.otf;
+#pragma unroll 1
+    while (p[0]) {
+        Factor f;
+        if (stream) ldg_factor_stream(f, p[0]);
+        else ldg_factor(f, p[0]);
+        mul_factor<F>(x, x, f);
+        p[0] = p[1];
+        p[1] = p[2];
+        p[2] = p[3];
+        p[3] = nullptr;
     }
-    if (a.fd) {
-        ldg_elem(g, a.fd + 2 * size_t(d));
-        mul_call<F>(f, f, g);
-    }
-    return true;
+    st_elem(a.out + 2 * tile_dst(a, tile, d, cc), x);
 }
 
 // Issue (without waiting) the 16-byte copies of one tile into shared memory:
@@ -202,8 +216,8 @@ __device__ __forceinline__ void issue_tile_load(const PassArgs &a, uint4 *smem, 
             uint32_t d = e0 >> lc;
             const uint4 *src = a.in + 2 * tile_src(a, tile, d, cc) + half;
             const size_t sstep = size_t(2 * dstep) << a.lo_bits;
-            if ((dstep & 15u) == 0) {
-                // rows d, d + dstep, ... agree in their low four bits, so they
+            if ((dstep & 31u) == 0) {
+                // rows d, d + dstep, ... agree in their low five bits, so they
                 // share the swizzle term and their slots step by dstep too
                 uint32_t sa = sbase + 16u * smem_slot(cc, d, K, lc);
                 for (uint32_t k = 0; k < iters; k++, sa += 16u * dstep, src += sstep)
@@ -243,209 +257,166 @@ __device__ __forceinline__ void issue_tile_load(const PassArgs &a, uint4 *smem, 
     }
 }
 
-// Process one tile with `nthreads` threads of the block (threads at or beyond
-// nthreads only take part in the barriers).  PRELOADED: the caller has
-// already copied the tile into `smem` and synchronised the block.  PAIR: let a
-// thread's two butterflies of one row pair share their twiddle (below).
-template <class F, int ILP, bool PRELOADED = false, bool SHFL = false, bool PAIR = true>
-__device__ __forceinline__ void run_tile(const PassArgs &a, uint4 *smem, uint32_t tile,
-                                         uint32_t nthreads) {
+// The sub-transform's twiddles in shared memory: the N/2 factors w_N^e in four
+// planes of N/2 16-byte quarters, entry e at slot tab_slot(e).  The slot's low
+// three bits fold in the higher ones, so eight entries at any power-of-two
+// stride lie in different bank groups.  (Read from global memory instead, they
+// missed L1 half the time and were two thirds of the load/store wavefronts.)
+__host__ __device__ __forceinline__ uint32_t tab_slot(uint32_t e) {
+    return e ^ (((e >> 3) ^ (e >> 6) ^ (e >> 9)) & 7u);
+}
+
+// entries of the table of a 2^K-point sub-transform
+__host__ __device__ constexpr uint32_t tab_entries(uint32_t K) { return K > 1 ? 1u << (K - 1) : 1u; }
+
+// issue (without waiting) the copies of the table, which is laid out in global
+// memory as in shared memory
+__device__ __forceinline__ void issue_table_load(const PassArgs &a, uint4 *tab) {
+    const uint32_t units = 4 * tab_entries(a.K);
+    for (uint32_t u = threadIdx.x; u < units; u += blockDim.x) cp_async16(tab + u, a.w_stage + u);
+}
+
+// the factor at table slot s (h = entries)
+__device__ __forceinline__ void lds_factor(Factor &f, const uint4 *tab, uint32_t h, uint32_t s) {
+    lds_elem(f.w, tab, tab + h, s);
+    lds_elem(f.wq, tab + 2 * h, tab + 3 * h, s);
+}
+
+// How a tile's stages run: two at a time, four elements a thread (radix 4), or
+// one by one, one butterfly a thread (radix 2); or either by the thread count.
+enum Steps { RADIX4 = 1, RADIX2 = 2, EITHER = 3 };
+
+// x <- x + y, t = x - y + r (for the product): the sum and lazy difference of
+// a butterfly
+template <class F>
+__device__ __forceinline__ void sum_diff(uint32_t x[8], uint32_t t[8], const uint32_t y[8]) {
+    sub_lazy<F>(t, x, y);
+    add<F>(x, x, y);
+}
+
+// One stage, pairs at distance h, one butterfly after the other.
+template <class F>
+__device__ __forceinline__ void radix2_stage(uint4 *s_lo, uint4 *s_hi, const uint4 *tab, uint32_t h,
+                                             uint32_t K, uint32_t lc, uint32_t tid,
+                                             uint32_t nthreads) {
+    const uint32_t N = 1u << K, CN = N << lc, step = row_slot(h);
+    const uint32_t shift = K - 1 - (31 - __clz(h));  // entry j 2^stage
+    for (uint32_t bk = tid; tid < nthreads && bk < (CN >> 1); bk += nthreads) {
+        const uint32_t cc = bk >> (K - 1), b = bk & ((N >> 1) - 1), j = b & (h - 1);
+        const uint32_t s0 = smem_slot(cc, ((b ^ j) << 1) | j, K, lc), s1 = s0 ^ step;
+        uint32_t x[8], y[8], t[8];
+        Factor w;
+        lds_elem(x, s_lo, s_hi, s0);
+        lds_elem(y, s_lo, s_hi, s1);
+        lds_factor(w, tab, N >> 1, tab_slot(j << shift));
+        sum_diff<F>(x, t, y);
+        mul_factor<F>(t, t, w);
+        sts_elem(s_lo, s_hi, s0, x);
+        sts_elem(s_lo, s_hi, s1, t);
+    }
+}
+
+// Process one tile, copied to `buf` with the table in `tab` (the block has
+// synchronised since), with `nthreads` threads of the block (threads at or
+// beyond nthreads only take part in the barriers).  The block does not
+// synchronise at the end: `buf` may be written again after a barrier.
+template <class F, Steps STEPS>
+__device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, uint4 *buf,
+                                         uint32_t tile, uint32_t nthreads) {
     const uint32_t K = a.K, lc = a.log_cols;
     const uint32_t N = 1u << K;
     const uint32_t C = 1u << lc;
     const uint32_t CN = C << K;
-    uint4 *s_lo = smem;
-    uint4 *s_hi = smem + CN;
+    uint4 *s_lo = buf;
+    uint4 *s_hi = buf + CN;
     const uint32_t tid = threadIdx.x;
     const bool active = tid < nthreads;
 
-    // ---- load (columns fastest for strided passes, rows fastest for the last)
-    if (PRELOADED) {
-    } else if (!a.pre && !a.pw_b) {
-        issue_tile_load(a, smem, tile, nthreads);
-        cp_async_wait_all();
-    } else {
+    // ---- input factors
+    if (a.pre || a.pw_b) {
+#pragma unroll 1
         for (uint32_t e = tid; active && e < CN; e += nthreads) {
             uint32_t d, cc;
             if (a.last) { d = e & (N - 1); cc = e >> K; }
             else        { cc = e & (C - 1); d = e >> lc; }
-            const size_t g = tile_src(a, tile, d, cc);
-            uint32_t x[8], f[8];
-            ld_elem_cg(x, a.in + 2 * g);
+            const uint32_t s = smem_slot(cc, d, K, lc);
+            uint32_t x[8];
+            lds_elem(x, s_lo, s_hi, s);
             if (a.pw_b) {
-                ld_elem_cg(f, a.pw_b + 2 * g);
-                mul_call<F>(x, x, f);
-                ld_elem_cg(f, a.pw_c + 2 * g);
-                sub<F>(x, x, f);
+                const size_t g = tile_src(a, tile, d, cc);
+                uint32_t v[8], u[8];
+                ld_elem_cg(v, a.pw_b + 2 * g);
+                ld_elem_cg(u, a.pw_c + 2 * g);
+                mul<F>(x, x, v);
+                sub<F>(x, x, u);
             }
             if (a.pre) {
-                ldg_elem(f, a.pre + 2 * size_t(d));
-                mul_call<F>(x, x, f);
+                Factor f;
+                ldg_factor(f, a.pre + 4 * size_t(d));
+                mul_factor<F>(x, x, f);
             }
-            sts_elem(s_lo, s_hi, smem_slot(cc, d, K, lc), x);
-        }
-    }
-    if (!PRELOADED) __syncthreads();
-
-    // ---- stages 0 .. K-3: radix-2 butterflies through shared memory.  Each
-    // thread takes ILP independent butterflies per step (every thread owns at
-    // least two per stage: nthreads <= C*N/4), so the carry chains and loads of
-    // one overlap with the other's product.
-    // SHFL: the stages with pair distance 16, 8 and 4 run in registers with
-    // warp shuffles (below) instead of through shared memory
-    const bool shfl_tail = SHFL && K >= 6 && nthreads >= 32;
-    // (K < 3: no loop stages; K - 2 must not wrap around)
-    const uint32_t s_end = shfl_tail ? K - 5 : (K > 2 ? K - 2 : 0u);
-    for (uint32_t s = 0; s < s_end; s++) {
-        const uint32_t lh = K - 1 - s;
-        const uint32_t h = 1u << lh;
-        const uint4 *ws = a.w_stage + 2 * size_t(N - 2 * h);
-        // slot of row i0 + h from that of row i0 (bit lh of i0 is clear): the
-        // swizzle term changes only when lh = 3
-        const uint32_t step = K < 3 ? h : (h ^ (lh == 3 ? 7u : 0u));
-        if constexpr (ILP == 0) {
-            // software-pipelined: the product of one butterfly overlaps the
-            // loads and add/subtract of the next (every thread owns >= 2)
-            uint32_t x[8], t[8], w[8], s0, s1;
-            auto prepare = [&](uint32_t bk, uint32_t px[8], uint32_t pt[8], uint32_t pw[8],
-                               uint32_t &q0, uint32_t &q1) {
-                const uint32_t cc = bk >> (K - 1);
-                const uint32_t b = bk & ((N >> 1) - 1);
-                const uint32_t j = b & (h - 1);
-                const uint32_t i0 = ((b >> lh) << (lh + 1)) | j;
-                q0 = smem_slot(cc, i0, K, lc);
-                q1 = q0 ^ step;
-                uint32_t py[8];
-                lds_elem(px, s_lo, s_hi, q0);
-                lds_elem(py, s_lo, s_hi, q1);
-                ldg_elem(pw, ws + 2 * size_t(j));
-                sub_lazy<F>(pt, px, py);
-                add<F>(px, px, py);
-            };
-            if (active) prepare(tid, x, t, w, s0, s1);
-            for (uint32_t bg = tid; active && bg < (CN >> 1); bg += nthreads) {
-                const uint32_t nb = bg + nthreads;
-                uint32_t x2[8], t2[8], w2[8], n0 = 0, n1 = 0;
-                if (nb < (CN >> 1)) prepare(nb, x2, t2, w2, n0, n1);
-                uint32_t y[8];
-                mul<F>(y, w, t);
-                sts_elem(s_lo, s_hi, s0, x);
-                sts_elem(s_lo, s_hi, s1, y);
-#pragma unroll
-                for (int k = 0; k < 8; k++) {
-                    x[k] = x2[k];
-                    t[k] = t2[k];
-                    w[k] = w2[k];
-                }
-                s0 = n0;
-                s1 = n1;
-            }
-        } else if (PAIR && ILP == 1 && lc >= 1 && (CN >> 1) == 2 * nthreads) {
-            // Each thread owns two butterflies, bk = tid and tid + C N/4: the
-            // same row pair in columns cc and cc + C/2, so one twiddle serves
-            // both and the second pair's slot is the first's moved by C/2
-            // columns, its swizzle term flipped in bit 2.
-            if (active) {
-                const uint32_t cc = tid >> (K - 1);
-                const uint32_t b = tid & ((N >> 1) - 1);
-                const uint32_t j = b & (h - 1);
-                const uint32_t i0 = ((b >> lh) << (lh + 1)) | j;
-                const uint32_t q0 = smem_slot(cc, i0, K, lc);
-                const uint32_t q0b = (q0 + ((C >> 1) << K)) ^ (K >= 3 ? 4u : 0u);
-                uint32_t w[8];
-                ldg_elem(w, ws + 2 * size_t(j));
-#pragma unroll
-                for (int q = 0; q < 2; q++) {
-                    const uint32_t a0 = q ? q0b : q0;
-                    uint32_t x[8], y[8], t[8];
-                    lds_elem(x, s_lo, s_hi, a0);
-                    lds_elem(y, s_lo, s_hi, a0 ^ step);
-                    sub_lazy<F>(t, x, y);
-                    add<F>(x, x, y);
-                    mul<F>(y, w, t);
-                    sts_elem(s_lo, s_hi, a0, x);
-                    sts_elem(s_lo, s_hi, a0 ^ step, y);
-                }
-            }
-        } else {
-        for (uint32_t bg = tid; active && bg < (CN >> 1); bg += ILP * nthreads) {
-            constexpr int IL = ILP > 0 ? ILP : 1;
-            uint32_t x[IL][8], y[IL][8], w[IL][8], t[IL][8], s0[IL], s1[IL];
-#pragma unroll
-            for (int k = 0; k < IL; k++) {
-                const uint32_t bk = bg + k * nthreads;
-                const uint32_t cc = bk >> (K - 1);
-                const uint32_t b = bk & ((N >> 1) - 1);
-                const uint32_t j = b & (h - 1);
-                const uint32_t i0 = ((b >> lh) << (lh + 1)) | j;
-                s0[k] = smem_slot(cc, i0, K, lc);
-                s1[k] = s0[k] ^ step;
-                lds_elem(x[k], s_lo, s_hi, s0[k]);
-                lds_elem(y[k], s_lo, s_hi, s1[k]);
-                ldg_elem(w[k], ws + 2 * size_t(j));
-            }
-#pragma unroll
-            for (int k = 0; k < IL; k++) {
-                sub_lazy<F>(t[k], x[k], y[k]);
-                add<F>(x[k], x[k], y[k]);
-            }
-#pragma unroll
-            for (int k = 0; k < IL; k++) mul<F>(y[k], w[k], t[k]);
-#pragma unroll
-            for (int k = 0; k < IL; k++) {
-                sts_elem(s_lo, s_hi, s0[k], x[k]);
-                sts_elem(s_lo, s_hi, s1[k], y[k]);
-            }
-        }
+            sts_elem(s_lo, s_hi, s, x);
         }
         __syncthreads();
     }
 
-    if constexpr (SHFL) {
-        if (shfl_tail) {
-            // A warp holds the 64 rows of one group (2 per lane) for the stages
-            // with pair distance h = 16, 8, 4.  At distance 2^lh lane L holds
-            // the pair (d, d + 2^lh), d = L with a zero inserted at bit lh; for
-            // the next distance, lanes L and L ^ 2^(lh-1) exchange one element
-            // (the one the partner's next pair needs) with 8 shuffles.
-            const uint32_t lane = tid & 31u, warp = tid >> 5, nwarps = nthreads >> 5;
-            const uint32_t groups = CN >> 6;
-            for (uint32_t gi = warp; active && gi < groups; gi += nwarps) {
-                const uint32_t cc = gi >> (K - 6), base = (gi & ((N >> 6) - 1)) << 6;
-                uint32_t d0 = ((lane >> 4) << 5) | (lane & 15u);
-                uint32_t x[8], y[8];
-                lds_elem(x, s_lo, s_hi, smem_slot(cc, base + d0, K, lc));
-                lds_elem(y, s_lo, s_hi, smem_slot(cc, base + d0 + 16, K, lc));
-                for (uint32_t lh = 4; lh >= 2; lh--) {
-                    const uint32_t h = 1u << lh;
-                    uint32_t w[8], t[8];
-                    ldg_elem(w, a.w_stage + 2 * (size_t(N - 2 * h) + (d0 & (h - 1))));
-                    sub_lazy<F>(t, x, y);
-                    add<F>(x, x, y);
-                    mul<F>(y, w, t);
-                    if (lh > 2) {
-                        const uint32_t m = h >> 1;
-                        const bool beta = (lane >> (lh - 1)) & 1u;
-#pragma unroll
-                        for (int k = 0; k < 8; k++) {
-                            const uint32_t r = __shfl_xor_sync(0xffffffffu, beta ? x[k] : y[k], m);
-                            if (beta) x[k] = r;
-                            else y[k] = r;
-                        }
-                        d0 = ((lane >> (lh - 1)) << lh) | (lane & (m - 1));
-                    }
-                }
-                sts_elem(s_lo, s_hi, smem_slot(cc, base + d0, K, lc), x);
-                sts_elem(s_lo, s_hi, smem_slot(cc, base + d0 + 4, K, lc), y);
-            }
+    // ---- stages 0 .. K-3
+    if (STEPS == RADIX2 || (STEPS == EITHER && nthreads > (CN >> 2))) {
+        for (uint32_t h = N >> 1; h >= 4; h >>= 1) {
+            radix2_stage<F>(s_lo, s_hi, tab, h, K, lc, tid, nthreads);
             __syncthreads();
+        }
+    } else if (K > 2) {
+        uint32_t q = N >> 2;  // distance of a radix-4 step's rows
+        if (K & 1u) {
+            radix2_stage<F>(s_lo, s_hi, tab, N >> 1, K, lc, tid, nthreads);
+            __syncthreads();
+            q >>= 1;
+        }
+        uint32_t shift = K & 1u;  // the step's first stage: entries j 2^shift and (j + q) 2^shift
+        for (; q > 1; q >>= 2, shift += 2) {
+            // rows i0 + {0, q, 2q, 3q}: the stage of distance 2q, then of distance q
+            const uint32_t x1 = row_slot(q), x2 = row_slot(2 * q), xt = tab_slot(q << shift);
+            for (uint32_t g = tid; active && g < (CN >> 2); g += nthreads) {
+                const uint32_t cc = g >> (K - 2), b = g & ((N >> 2) - 1), j = b & (q - 1);
+                const uint32_t s0 = smem_slot(cc, ((b ^ j) << 2) | j, K, lc);
+                const uint32_t ta = tab_slot(j << shift), tb = tab_slot(j << (shift + 1));
+                uint32_t v0[8], v1[8], v2[8], v3[8], t[8];
+                Factor w;
+                lds_elem(v0, s_lo, s_hi, s0);
+                lds_elem(v2, s_lo, s_hi, s0 ^ x2);
+                lds_factor(w, tab, N >> 1, ta);
+                sum_diff<F>(v0, t, v2);
+                mul_factor<F>(v2, t, w);
+                lds_elem(v1, s_lo, s_hi, s0 ^ x1);
+                lds_elem(v3, s_lo, s_hi, s0 ^ x1 ^ x2);
+                lds_factor(w, tab, N >> 1, ta ^ xt);
+                sum_diff<F>(v1, t, v3);
+                mul_factor<F>(v3, t, w);
+                lds_factor(w, tab, N >> 1, tb);
+                sum_diff<F>(v0, t, v1);
+                sts_elem(s_lo, s_hi, s0, v0);
+                mul_factor<F>(v1, t, w);
+                sts_elem(s_lo, s_hi, s0 ^ x1, v1);
+                sum_diff<F>(v2, t, v3);
+                sts_elem(s_lo, s_hi, s0 ^ x2, v2);
+                mul_factor<F>(v3, t, w);
+                sts_elem(s_lo, s_hi, s0 ^ x1 ^ x2, v3);
+            }
+            // at q <= 32 a warp's groups, 32 consecutive ones, are made of rows
+            // of its own, at this step and the next: only the last step (columns
+            // fastest) reads another warp's
+            if (q > 32 || q == 4) __syncthreads();
+            else __syncwarp();
         }
     }
 
-    // ---- last two stages as radix-4 on rows d0..d0+3 (columns fastest)
+    // ---- last two stages as radix-4 on rows d0..d0+3, factors and store
+    // (columns fastest: C-element runs in global memory)
+    const bool scaled = a.last ? a.post != nullptr : true;
     if (K >= 2) {
-        uint32_t w4[8];
-        ldg_elem(w4, a.w_stage + 2 * size_t(N - 3));  // w_N^(2^(K-2)) = w_4
+        Factor w4;
+        lds_factor(w4, tab, N >> 1, tab_slot(N >> 2));  // w_N^(N/4) = w_4
         for (uint32_t qd = tid; active && qd < (CN >> 2); qd += nthreads) {
             const uint32_t cc = qd & (C - 1);
             const uint32_t d0 = (qd >> lc) << 2;
@@ -462,20 +433,33 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, uint4 *smem, uint32_
             add<F>(x0, x0, x2);
 #pragma unroll
             for (int k = 0; k < 8; k++) x2[k] = t[k];
-            sub_lazy<F>(t, x1, x3);
-            add<F>(x1, x1, x3);
-            mul<F>(x3, w4, t);
+            sum_diff<F>(x1, t, x3);
+            mul_factor<F>(x3, t, w4);
             // stage K-1: pairs (0,1), (2,3), twiddle 1
             sub<F>(t, x0, x1);
             add<F>(x0, x0, x1);
-#pragma unroll
-            for (int k = 0; k < 8; k++) x1[k] = t[k];
+            if (!scaled) {
+                st_elem(a.out + 2 * tile_dst(a, tile, d0, cc), x0);
+                st_elem(a.out + 2 * tile_dst(a, tile, d0 + 1, cc), t);
+                sub<F>(t, x2, x3);
+                add<F>(x2, x2, x3);
+                st_elem(a.out + 2 * tile_dst(a, tile, d0 + 2, cc), x2);
+                st_elem(a.out + 2 * tile_dst(a, tile, d0 + 3, cc), t);
+                continue;
+            }
+            // through the thread's own slots into a loop with one product
+            sts_elem(s_lo, s_hi, s0, x0);
+            sts_elem(s_lo, s_hi, s1, t);
             sub<F>(t, x2, x3);
             add<F>(x2, x2, x3);
-            sts_elem(s_lo, s_hi, s0, x0);
-            sts_elem(s_lo, s_hi, s1, x1);
             sts_elem(s_lo, s_hi, s2, x2);
             sts_elem(s_lo, s_hi, s3, t);
+#pragma unroll 1
+            for (uint32_t i = 0; i < 4; i++) {
+                uint32_t x[8];
+                lds_elem(x, s_lo, s_hi, s0 ^ i);
+                scale_and_store<F>(x, a, tile, d0 + i, cc);
+            }
         }
     } else {
         // N = 2: one radix-2 butterfly per column
@@ -488,19 +472,14 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, uint4 *smem, uint32_
             add<F>(x0, x0, x1);
             sts_elem(s_lo, s_hi, s0, x0);
             sts_elem(s_lo, s_hi, s1, t);
+#pragma unroll 1
+            for (uint32_t i = 0; i < 2; i++) {
+                uint32_t x[8];
+                lds_elem(x, s_lo, s_hi, s0 + i);
+                scale_and_store<F>(x, a, tile, i, cc);
+            }
         }
     }
-    __syncthreads();
-
-    // ---- scale and store (columns fastest: C-element runs in global memory)
-    for (uint32_t e = tid; active && e < CN; e += nthreads) {
-        const uint32_t cc = e & (C - 1), d = e >> lc;
-        uint32_t x[8], f[8];
-        lds_elem(x, s_lo, s_hi, smem_slot(cc, d, K, lc));
-        if (out_factor<F>(f, a, tile, d, cc)) mul<F>(x, x, f);
-        st_elem(a.out + 2 * tile_dst(a, tile, d, cc), x);
-    }
-    __syncthreads();
 }
 
 // threads per block for a tile of C x 2^K elements: one per radix-4 group,
@@ -518,70 +497,32 @@ __host__ __device__ constexpr uint32_t pass_threads_for(uint32_t K, uint32_t lc,
                                                            : pass_threads(K, lc);
 }
 
-// Schedule variants (the plan's `ilp` option):
-//   1: one butterfly per thread per stage step, registers for 3 blocks of 256
-//   2: two interleaved butterflies per thread, registers for 2 blocks
-//   3: one butterfly per thread, registers for 4 blocks (tiles of <= 1024
-//      elements so four fit in shared memory)
-//   4: software-pipelined stage loop (the product of one butterfly overlaps
-//      the loads and add/subtract of the next), registers for 2 blocks
-//   5: as 3 with twice the threads per tile (one butterfly per thread per
-//      stage; half the threads idle in the radix-4 epilogue): more warps in
-//      flight for transforms too small to fill the GPU
-//   6: as 3 with two tile buffers: the next tile's loads overlap this tile's
-//      stages (twice the shared memory per block)
-//   7: as 1 with the stages of pair distance 16, 8 and 4 in registers, the
-//      partners exchanged by warp shuffles (digits of 6 bits or more)
-template <int V> struct PassVariant;
-template <> struct PassVariant<1> { static constexpr int ILP = 1, MIN_BLOCKS = 3; };
-template <> struct PassVariant<2> { static constexpr int ILP = 2, MIN_BLOCKS = 2; };
-template <> struct PassVariant<3> { static constexpr int ILP = 1, MIN_BLOCKS = 4; };
-template <> struct PassVariant<4> { static constexpr int ILP = 0, MIN_BLOCKS = 2; };  // pipelined
-template <> struct PassVariant<5> { static constexpr int ILP = 1, MIN_BLOCKS = 4; };  // 2x threads
-template <> struct PassVariant<6> { static constexpr int ILP = 1, MIN_BLOCKS = 4; };  // 2 buffers
-template <> struct PassVariant<7> { static constexpr int ILP = 1, MIN_BLOCKS = 3; };  // shuffles
-
-template <class F, int V>
-__global__ void __launch_bounds__(256, PassVariant<V>::MIN_BLOCKS) ntt_pass_kernel(const PassArgs a) {
+// One pass.  MIN_BLOCKS: blocks of 256 threads an SM the register budget is
+// for (2: 128 registers, 3: 80, 4: 64).
+template <class F, int MIN_BLOCKS, Steps STEPS>
+__global__ void __launch_bounds__(256, MIN_BLOCKS) ntt_pass_kernel(const PassArgs a) {
     extern __shared__ uint4 smem[];
+    // Two tile buffers when the block has more than one tile: the copies of its
+    // next tile are in flight while the current one is computed.
+    const uint32_t CN = 1u << (a.K + a.log_cols);
+    uint4 *tab = smem, *buf = smem + 4 * tab_entries(a.K);
+    uint32_t tile = blockIdx.x;
+    issue_table_load(a, tab);  // (a plan's table: no pass writes it)
     // Passes after the first are launched as programmatic dependents of the
     // pass before, and wait here until that pass has completed and its writes
     // are visible (launched without that attribute, the wait returns at once).
     // A block lets the next pass launch when it starts its last tile, so the
     // next pass's blocks take SM places only as this grid winds down.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (V != 6 || a.pre || a.pw_b) {
-        for (uint32_t tile = blockIdx.x; tile < a.num_tiles; tile += gridDim.x) {
-            if (tile + gridDim.x >= a.num_tiles)
-                asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            run_tile<F, PassVariant<V>::ILP, false, V == 7>(a, smem, tile, blockDim.x);
-        }
-        return;
-    }
-    // Variant 6: two tile buffers.  The copies of the block's next tile are in
-    // flight (cp.async group) while the current tile's stages run, so a tile's
-    // load latency overlaps the previous tile's arithmetic within the block.
-    // The buffer a load goes to was last used by the tile before, which ended
-    // with a block barrier.
-    const uint32_t CN = 1u << (a.K + a.log_cols);
-    uint32_t tile = blockIdx.x;
-    if (tile >= a.num_tiles) return;
-    issue_tile_load(a, smem, tile, blockDim.x);
-    cp_async_commit();
-    uint32_t cur = 0;
-    for (; tile < a.num_tiles; tile += gridDim.x) {
-        const uint32_t next = tile + gridDim.x;
-        if (next >= a.num_tiles) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (next < a.num_tiles) {
-            issue_tile_load(a, smem + (cur ^ 1u) * 2 * CN, next, blockDim.x);
-            cp_async_commit();
-            cp_async_wait_group<1>();
-        } else {
-            cp_async_wait_group<0>();
-        }
+    if (tile < a.num_tiles) issue_tile_load(a, buf, tile, blockDim.x);
+    for (uint32_t cur = 0; tile < a.num_tiles; tile += gridDim.x, cur ^= 2 * CN) {
+        cp_async_wait_all();
+        // the tile is there, and every thread is done with the other buffer
         __syncthreads();
-        run_tile<F, 1, true>(a, smem + cur * 2 * CN, tile, blockDim.x);
-        cur ^= 1u;
+        const uint32_t next = tile + gridDim.x;
+        if (next < a.num_tiles) issue_tile_load(a, buf + (cur ^ (2 * CN)), next, blockDim.x);
+        else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        run_tile<F, STEPS>(a, tab, buf + cur, tile, blockDim.x);
     }
 }
 

@@ -60,6 +60,7 @@ struct HostField {
     uint32_t rp = 0;   // -p^-1 mod 2^32
     E8 one{};          // R mod p
     E8 r2{};           // R^2 mod p
+    E8 ninv{};         // -p^-1 mod R
     uint32_t gen = 0;  // multiplicative generator (plain)
     int s = 0;         // 2-adicity
     E8 gen_m{};        // generator, Montgomery form
@@ -125,6 +126,33 @@ E8 hmul(const HostField &F, const E8 &a, const E8 &b) {
     return r;
 }
 
+// low 256 bits of a b
+E8 hmul_low(const E8 &a, const E8 &b) {
+    E8 z{};
+    for (int i = 0; i < 8; i++) {
+        uint64_t carry = 0;
+        for (int j = 0; i + j < 8; j++) {
+            const uint64_t v = uint64_t(a[i]) * b[j] + z[i + j] + carry;
+            z[i + j] = uint32_t(v);
+            carry = v >> 32;
+        }
+    }
+    return z;
+}
+
+// A factor table entry of w, given in Montgomery form as m = w R mod p: the
+// integer w and floor(w R / p).  w R = floor(w R / p) p + m, so modulo R the
+// quotient is -m p^-1, and it is below R.
+struct HFactor {
+    E8 w, wq;
+};
+
+HFactor hfactor(const HostField &F, const E8 &m) {
+    E8 one{};
+    one[0] = 1;
+    return {hmul(F, m, one), hmul_low(m, F.ninv)};
+}
+
 E8 hsub(const HostField &F, const E8 &a, const E8 &b) {
     E8 r;
     if (sub8(r, a, b)) add8(r, r, F.p);
@@ -186,6 +214,16 @@ HostField make_field(uint32_t gen) {
         x = y;
     }
     F.r2 = x;
+    // -p^-1 mod R by Newton's iteration: y <- y (2 + p y) for y = -p^-1
+    E8 y{};
+    y[0] = F.rp;
+    for (int bits = 32; bits < 256; bits *= 2) {
+        E8 two{}, t = hmul_low(F.p, y);
+        two[0] = 2;
+        add8(t, t, two);
+        y = hmul_low(y, t);
+    }
+    F.ninv = y;
     F.gen = gen;
     E8 pm1, onep{};
     onep[0] = 1;
@@ -230,10 +268,16 @@ uint32_t rev_bits(uint32_t x, int bits) {
 // beyond the slab share its last word.
 constexpr int STATUS_WORDS = 1024;
 
+// the largest twiddle table (64 KiB, K = 11) and two tile buffers of 64 KiB
+constexpr int PASS_MAX_SMEM = 192 * 1024;
+// a batch launch takes shared memory in steps of 4 KiB, at most the largest
+// table and one tile buffer
+constexpr int BATCH_SMEM_STEP = 4 * 1024, BATCH_SMEM_STEPS = 32;
+
 struct DeviceInfo {
     int sms = 0;
-    // batch kernel occupancy per field for 2^(10+i) bytes of shared memory
-    int batch_blocks_per_sm[NUM_FIELDS][8] = {};
+    // batch kernel occupancy per field for i steps of shared memory
+    int batch_blocks_per_sm[NUM_FIELDS][BATCH_SMEM_STEPS + 1] = {};
     bool init = false;
     uint32_t *status_slab = nullptr;             // STATUS_WORDS sticky error words
     std::map<uintptr_t, int> status_of_stream;   // stream handle -> word index
@@ -256,14 +300,15 @@ zkntt_status device_info(DeviceInfo **out) {
             for (int ilp = 1; ilp <= NUM_VARIANTS; ilp++)
                 ZK_CHECK(cudaFuncSetAttribute(field_kernels(f).pass[ilp],
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (ilp == 6 ? 128 : 64) * 1024));
+                                              PASS_MAX_SMEM));
         for (int f = 0; f < NUM_FIELDS; f++) {
             ZK_CHECK(cudaFuncSetAttribute(batch_kernel_ptr(f),
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-            for (int i = 0; i < 7; i++) {
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          BATCH_SMEM_STEP * BATCH_SMEM_STEPS));
+            for (int i = 0; i <= BATCH_SMEM_STEPS; i++) {
                 ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                     &d.batch_blocks_per_sm[f][i], batch_kernel_ptr(f), BATCH_THREADS,
-                    size_t(1024) << i));
+                    size_t(BATCH_SMEM_STEP) * i));
                 d.batch_blocks_per_sm[f][i] = std::max(d.batch_blocks_per_sm[f][i], 1);
             }
         }
@@ -354,7 +399,18 @@ zkntt_status dalloc(zkntt_plan_s *P, uint4 **out, size_t elems) {
     return ZKNTT_OK;
 }
 
-zkntt_status upload(zkntt_plan_s *P, uint4 **out, const std::vector<E8> &v) {
+// values in Montgomery form, uploaded as factors
+zkntt_status upload_factors(zkntt_plan_s *P, const HostField &F, uint4 **out,
+                            const std::vector<E8> &v) {
+    std::vector<HFactor> f;
+    f.reserve(v.size());
+    for (const E8 &m : v) f.push_back(hfactor(F, m));
+    zkntt_status s = dalloc(P, out, 2 * v.size());
+    if (s != ZKNTT_OK) return s;
+    return from_cuda(cudaMemcpy(*out, f.data(), f.size() * 64, cudaMemcpyHostToDevice));
+}
+
+zkntt_status upload(zkntt_plan_s *P, const HostField &, uint4 **out, const std::vector<E8> &v) {
     zkntt_status s = dalloc(P, out, v.size());
     if (s != ZKNTT_OK) return s;
     return from_cuda(cudaMemcpy(*out, v.data(), v.size() * 32, cudaMemcpyHostToDevice));
@@ -409,35 +465,45 @@ int default_log_cols(int K, int span_bits) {
     return std::max(0, std::min(lc, span_bits));
 }
 
+NegInv neg_inv(int field) {
+    NegInv n;
+    memcpy(n.v, host_field(field).ninv.data(), 32);
+    return n;
+}
+
 zkntt_status launch_gen_twiddle(int field, uint4 *out, int K, int lo_bits, const uint4 *w_hi,
                                 const uint4 *w_lo, int split, const uint4 *fl, const uint4 *fd,
                                 int sms) {
     const FieldKernels &kk = field_kernels(field);
     uint32_t uK = K, ulo = lo_bits, usp = split;
-    void *args[] = {&out, &uK, &ulo, &w_hi, &w_lo, &usp, &fl, &fd};
+    NegInv ni = neg_inv(field);
+    void *args[] = {&out, &uK, &ulo, &w_hi, &w_lo, &usp, &fl, &fd, &ni};
     size_t total = size_t(1) << (K + lo_bits);
     return from_cuda(cudaLaunchKernel(kk.gen_twiddle, dim3(grid_for(total, 256, sms)), dim3(256),
                                       args, 0, nullptr));
 }
 
 zkntt_status launch_gen_powers(int field, uint4 *out, uint32_t count, const uint4 *hi,
-                               const uint4 *lo, int split, int sms) {
+                               const uint4 *lo, int split, bool factors, int sms) {
     const FieldKernels &kk = field_kernels(field);
-    uint32_t usp = split;
-    void *args[] = {&out, &count, &hi, &lo, &usp};
+    uint32_t usp = split, uf = factors;
+    NegInv ni = neg_inv(field);
+    void *args[] = {&out, &count, &hi, &lo, &usp, &uf, &ni};
     return from_cuda(cudaLaunchKernel(kk.gen_powers, dim3(grid_for(count, 256, sms)), dim3(256),
                                       args, 0, nullptr));
 }
 
-// split tables for base^e, e < 2^bits: lo[x] = base^x * scale, hi[y] = base^(y 2^split)
+// split tables for base^e, e < 2^bits: lo[x] = base^x * scale, hi[y] = base^(y 2^split),
+// in Montgomery form (what the table kernels read) or as factors
 zkntt_status split_tables(zkntt_plan_s *P, const HostField &F, const E8 &base, int bits,
-                          const E8 &scale, uint4 **hi, uint4 **lo, int *split) {
+                          const E8 &scale, bool factors, uint4 **hi, uint4 **lo, int *split) {
     int sp = (bits + 1) / 2;
     *split = sp;
-    zkntt_status s = upload(P, lo, powers(F, base, size_t(1) << sp, scale));
+    auto put = factors ? upload_factors : upload;
+    zkntt_status s = put(P, F, lo, powers(F, base, size_t(1) << sp, scale));
     if (s != ZKNTT_OK) return s;
     E8 step = hpow(F, base, uint64_t(1) << sp);
-    return upload(P, hi, powers(F, step, size_t(1) << (bits - sp), F.one));
+    return put(P, F, hi, powers(F, step, size_t(1) << (bits - sp), F.one));
 }
 
 zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
@@ -492,8 +558,8 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
     }
     const int p = P->passes;
     if (mode == ZKNTT_TWIDDLE_AUTO && p > 1) {
-        // Precomputed inter-pass tables (pass i: 2^(K_i + lo_bits_i) entries;
-        // pass 1's is n entries) unless they would not fit beside the input,
+        // Precomputed inter-pass tables (pass i: 2^(K_i + lo_bits_i) entries of
+        // 64 bytes; pass 1's is n entries) unless they would not fit beside the input,
         // output and scratch vectors in the device memory free now: then the
         // split-exponent tables (about 2 sqrt(n_i) entries) instead.
         size_t fr = 0, tot = 0;
@@ -501,7 +567,7 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         size_t tables = 0;
         for (int i = 0, hb = 0; i < p - 1; i++) {
             hb += k[i];
-            tables += size_t(32) << (L - hb + k[i]);
+            tables += size_t(64) << (L - hb + k[i]);
         }
         const size_t vectors = 3 * (size_t(32) << L);
         if (tables + vectors > fr) mode = ZKNTT_TWIDDLE_OTF;
@@ -544,26 +610,39 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         ps.num_tiles = last ? (uint32_t(1) << (ps.hi_bits - lc))
                             : (uint32_t(1) << (ps.hi_bits + ps.lo_bits - lc));
         ps.threads = int(pass_threads_for(uint32_t(ps.K), uint32_t(lc), ilp));
-        ps.smem = size_t(32) << (ps.K + lc);
-        if (ilp == 6) ps.smem *= 2;  // two tile buffers
+        // the twiddle table, and two tile buffers unless every block has one tile
+        const size_t tile_bytes = size_t(32) << (ps.K + lc);
+        const size_t table_bytes = size_t(64) * tab_entries(uint32_t(ps.K));
         int nb = 0;
-        ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &nb, field_kernels(P->field).pass[ps.ilp], ps.threads, ps.smem));
-        nb = std::max(nb, 1);
+        for (int buffers = 1; buffers <= 2; buffers++) {
+            ps.smem = table_bytes + buffers * tile_bytes;
+            ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &nb, field_kernels(P->field).pass[ps.ilp], ps.threads, ps.smem));
+            nb = std::max(nb, 1);
+            if (ps.num_tiles <= uint64_t(nb) * dev->sms) break;
+        }
         ps.grid = int(std::min<uint64_t>(ps.num_tiles, uint64_t(nb) * dev->sms));
 
-        // sub-transform twiddles, stage-major: stage s holds w_N^(j 2^s) for
-        // j < N / 2^(s+1) at offset N - 2^(K-s)
+        // sub-transform twiddles w_N^e, e < N/2 (stage s uses w_N^(j 2^s))
         const E8 wn_i = hpow(F, w, uint64_t(1) << ps.hi_bits);          // root of order n_i
         const E8 wN = hpow(F, wn_i, uint64_t(1) << ps.lo_bits);         // root of order N_i
         {
-            const size_t N = size_t(1) << ps.K;
-            std::vector<E8> all = powers(F, wN, std::max<size_t>(1, N / 2), F.one);
-            std::vector<E8> st_tab;
-            st_tab.reserve(N);
-            for (int sidx = 0; sidx < ps.K; sidx++)
-                for (size_t j = 0; j < (N >> (sidx + 1)); j++) st_tab.push_back(all[j << sidx]);
-            st = upload(P, &ps.w_stage, st_tab);
+            // (in four planes of 16-byte quarters, as the kernels keep it in
+            // shared memory)
+            const uint32_t h = tab_entries(uint32_t(ps.K));
+            const std::vector<E8> all = powers(F, wN, h, F.one);
+            std::vector<uint32_t> planes(size_t(h) * 16);
+            for (uint32_t e = 0; e < h; e++) {
+                const HFactor f = hfactor(F, all[e]);
+                uint32_t q[16];
+                memcpy(q, f.w.data(), 32);
+                memcpy(q + 8, f.wq.data(), 32);
+                for (int p4 = 0; p4 < 4; p4++)
+                    memcpy(&planes[(size_t(p4) * h + tab_slot(e)) * 4], q + 4 * p4, 16);
+            }
+            st = dalloc(P, &ps.w_stage, 2 * size_t(h));
+            if (st != ZKNTT_OK) return st;
+            st = from_cuda(cudaMemcpy(ps.w_stage, planes.data(), size_t(h) * 64, cudaMemcpyHostToDevice));
             if (st != ZKNTT_OK) return st;
         }
 
@@ -578,25 +657,27 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         if (!last) {
             ps.tw_bits = ps.K + ps.lo_bits;
             const E8 scale = (i == 0) ? out_scale : F.one;
-            st = split_tables(P, F, wn_i, ps.tw_bits, scale, &ps.w_hi, &ps.w_lo, &ps.split_bits);
+            const bool otf = mode == ZKNTT_TWIDDLE_OTF;
+            st = split_tables(P, F, wn_i, ps.tw_bits, scale, otf, &ps.w_hi, &ps.w_lo, &ps.split_bits);
             if (st != ZKNTT_OK) return st;
             if (i == 0 && coset && !inverse) {
                 // column factor g^lo, lo < 2^lo_bits
                 uint4 *ghi, *glo;
                 int gsp;
-                st = split_tables(P, F, g, ps.lo_bits, F.one, &ghi, &glo, &gsp);
+                st = split_tables(P, F, g, ps.lo_bits, F.one, false, &ghi, &glo, &gsp);
                 if (st != ZKNTT_OK) return st;
-                st = dalloc(P, &ps.fl, size_t(1) << ps.lo_bits);
+                st = dalloc(P, &ps.fl, size_t(otf ? 2 : 1) << ps.lo_bits);
                 if (st != ZKNTT_OK) return st;
-                st = launch_gen_powers(P->field, ps.fl, uint32_t(1) << ps.lo_bits, ghi, glo, gsp, dev->sms);
+                st = launch_gen_powers(P->field, ps.fl, uint32_t(1) << ps.lo_bits, ghi, glo, gsp, otf,
+                                       dev->sms);
                 if (st != ZKNTT_OK) return st;
             }
             if (!phi.empty()) {
-                st = upload(P, &ps.fd, phi);
+                st = (otf ? upload_factors : upload)(P, F, &ps.fd, phi);
                 if (st != ZKNTT_OK) return st;
             }
             if (mode == ZKNTT_TWIDDLE_PRECOMP) {
-                st = dalloc(P, &ps.tw, size_t(1) << (ps.K + ps.lo_bits));
+                st = dalloc(P, &ps.tw, size_t(2) << (ps.K + ps.lo_bits));
                 if (st != ZKNTT_OK) return st;
                 st = launch_gen_twiddle(P->field, ps.tw, ps.K, ps.lo_bits, ps.w_hi, ps.w_lo,
                                         ps.split_bits, ps.fl, ps.fd, dev->sms);
@@ -611,14 +692,14 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
                 std::vector<E8> q(N, p == 1 ? out_scale : F.one);
                 if (!phi.empty())
                     for (size_t d = 0; d < N; d++) q[d] = hmul(F, q[d], phi[d]);
-                st = upload(P, &P->post, q);
+                st = upload_factors(P, F, &P->post, q);
                 if (st != ZKNTT_OK) return st;
             }
         }
         if (i == 0 && coset && !inverse) {
             // input row factor (g^(2^lo_bits))^d
             const E8 gs = hpow(F, g, uint64_t(1) << ps.lo_bits);
-            st = upload(P, &P->pre, powers(F, gs, size_t(1) << ps.K, F.one));
+            st = upload_factors(P, F, &P->pre, powers(F, gs, size_t(1) << ps.K, F.one));
             if (st != ZKNTT_OK) return st;
         }
     }
@@ -897,15 +978,18 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
     }
     cudaError_t e = cudaMemsetAsync(ctrl, 0, words * 4, s);
     if (e == cudaSuccess) {
-        // shared memory for the largest tile of the launch; occupancy comes from
+        // shared memory for the largest tile and table of the launch; occupancy comes from
         // the table built at device set-up (no query here: this path must stay
         // legal inside a stream capture)
-        size_t smem = 1024;
-        for (int k = 0; k < int(segs.size()); k++)
-            smem = std::max(smem, size_t(32) << (tab->seg[k].a.K + tab->seg[k].a.log_cols));
-        int si = 0;
-        while ((size_t(1024) << si) < smem) si++;
-        smem = size_t(1024) << si;
+        size_t tile_bytes = 0, table_bytes = 0;
+        for (int k = 0; k < int(segs.size()); k++) {
+            const PassArgs &a = tab->seg[k].a;
+            tile_bytes = std::max(tile_bytes, size_t(32) << (a.K + a.log_cols));
+            table_bytes = std::max(table_bytes, size_t(64) * tab_entries(a.K));
+        }
+        tab->table_units = uint32_t(table_bytes / 16);
+        const int si = int((tile_bytes + table_bytes + BATCH_SMEM_STEP - 1) / BATCH_SMEM_STEP);
+        const size_t smem = size_t(BATCH_SMEM_STEP) * si;
         // Resident blocks: at most what fits, and no more than splits the
         // widest dependency level into whole, equal waves -- a level of T tiles
         // over G blocks otherwise ends in a partial wave with most SMs idle
