@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, BATCH_MIN_BLOCKS)
         uint4 *buf = smem + tab.table_units;
         if (sg.a.w_stage != table) {
             table = sg.a.w_stage;
-            issue_table_load(sg.a, smem);
+            issue_table_load(sg.a, smem, BATCH_THREADS);
         }
         issue_tile_load(sg.a, buf, tile, nt);
         cp_async_wait_all();

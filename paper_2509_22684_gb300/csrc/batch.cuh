@@ -27,9 +27,9 @@ namespace zkntt {
 
 constexpr int BATCH_MAX_SEGMENTS = 160;
 constexpr uint32_t BATCH_THREADS = 256;
-// blocks per SM the register budget is compiled for (64 registers a thread)
+// blocks per SM the register budget is compiled for (80 registers a thread)
 #ifndef ZKNTT_BATCH_MIN_BLOCKS
-#define ZKNTT_BATCH_MIN_BLOCKS 4
+#define ZKNTT_BATCH_MIN_BLOCKS 3
 #endif
 constexpr int BATCH_MIN_BLOCKS = ZKNTT_BATCH_MIN_BLOCKS;
 // resident blocks per SM the tile-width policy counts as one wave

@@ -118,6 +118,144 @@ __device__ __forceinline__ void sub(uint32_t r[8], const uint32_t a[8], const ui
           "r"(F::P4 & mask), "r"(F::P5 & mask), "r"(F::P6 & mask), "r"(F::P7 & mask));
 }
 
+// ---------------------------------------------------------------------------
+// Residues in [0, 2r) ("loose"): inside a transform no value is brought below r;
+// the last pass does that once per output.  2r < 2^256 for the three fields; 4r
+// is too for BN254 and BLS12-377, not for BLS12-381.
+template <class F>
+struct Twice {
+    static constexpr uint32_t D0 = F::P0 << 1, D1 = (F::P1 << 1) | (F::P0 >> 31),
+                              D2 = (F::P2 << 1) | (F::P1 >> 31), D3 = (F::P3 << 1) | (F::P2 >> 31),
+                              D4 = (F::P4 << 1) | (F::P3 >> 31), D5 = (F::P5 << 1) | (F::P4 >> 31),
+                              D6 = (F::P6 << 1) | (F::P5 >> 31), D7 = (F::P7 << 1) | (F::P6 >> 31);
+    static constexpr bool SUM_FITS = F::P7 < 0x40000000u;  // 4r < 2^256
+};
+
+// r = a + b, less 2p unless below it: loose from loose
+template <class F>
+__device__ __forceinline__ void add_loose(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
+    using D = Twice<F>;
+    uint32_t s[8], u[8], mask, c = 0;
+    if constexpr (D::SUM_FITS)
+        asm("add.cc.u32  %0, %8, %16;\n\t"
+            "addc.cc.u32 %1, %9, %17;\n\t"
+            "addc.cc.u32 %2, %10, %18;\n\t"
+            "addc.cc.u32 %3, %11, %19;\n\t"
+            "addc.cc.u32 %4, %12, %20;\n\t"
+            "addc.cc.u32 %5, %13, %21;\n\t"
+            "addc.cc.u32 %6, %14, %22;\n\t"
+            "addc.u32    %7, %15, %23;"
+            : "=r"(s[0]), "=r"(s[1]), "=r"(s[2]), "=r"(s[3]), "=r"(s[4]), "=r"(s[5]), "=r"(s[6]),
+              "=r"(s[7])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
+              "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]),
+              "r"(b[7]));
+    else
+        asm("add.cc.u32  %0, %9, %17;\n\t"
+            "addc.cc.u32 %1, %10, %18;\n\t"
+            "addc.cc.u32 %2, %11, %19;\n\t"
+            "addc.cc.u32 %3, %12, %20;\n\t"
+            "addc.cc.u32 %4, %13, %21;\n\t"
+            "addc.cc.u32 %5, %14, %22;\n\t"
+            "addc.cc.u32 %6, %15, %23;\n\t"
+            "addc.cc.u32 %7, %16, %24;\n\t"
+            "addc.u32    %8, 0, 0;"
+            : "=r"(s[0]), "=r"(s[1]), "=r"(s[2]), "=r"(s[3]), "=r"(s[4]), "=r"(s[5]), "=r"(s[6]),
+              "=r"(s[7]), "=r"(c)
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
+              "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]),
+              "r"(b[7]));
+    // mask = c - borrow: all ones when the sum is below 2p (c = 0 and a borrow;
+    // a carry out always comes with a borrow, since a + b - 2p < 2^256)
+    asm("sub.cc.u32  %0, %9, %17;\n\t"
+        "subc.cc.u32 %1, %10, %18;\n\t"
+        "subc.cc.u32 %2, %11, %19;\n\t"
+        "subc.cc.u32 %3, %12, %20;\n\t"
+        "subc.cc.u32 %4, %13, %21;\n\t"
+        "subc.cc.u32 %5, %14, %22;\n\t"
+        "subc.cc.u32 %6, %15, %23;\n\t"
+        "subc.cc.u32 %7, %16, %24;\n\t"
+        "subc.u32    %8, %25, 0;"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
+          "=r"(u[7]), "=r"(mask)
+        : "r"(s[0]), "r"(s[1]), "r"(s[2]), "r"(s[3]), "r"(s[4]), "r"(s[5]), "r"(s[6]), "r"(s[7]),
+          "n"(D::D0), "n"(D::D1), "n"(D::D2), "n"(D::D3), "n"(D::D4), "n"(D::D5), "n"(D::D6),
+          "n"(D::D7), "r"(c));
+#pragma unroll
+    for (int i = 0; i < 8; i++) r[i] = u[i] ^ ((s[i] ^ u[i]) & mask);
+}
+
+// r = a - b, plus 2p if negative: loose from loose
+template <class F>
+__device__ __forceinline__ void sub_loose(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
+    using D = Twice<F>;
+    uint32_t mask, u[8];
+    asm("sub.cc.u32  %0, %9, %17;\n\t"
+        "subc.cc.u32 %1, %10, %18;\n\t"
+        "subc.cc.u32 %2, %11, %19;\n\t"
+        "subc.cc.u32 %3, %12, %20;\n\t"
+        "subc.cc.u32 %4, %13, %21;\n\t"
+        "subc.cc.u32 %5, %14, %22;\n\t"
+        "subc.cc.u32 %6, %15, %23;\n\t"
+        "subc.cc.u32 %7, %16, %24;\n\t"
+        "subc.u32    %8, 0, 0;"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
+          "=r"(u[7]), "=r"(mask)
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
+          "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7]));
+    asm("add.cc.u32  %0, %8, %16;\n\t"
+        "addc.cc.u32 %1, %9, %17;\n\t"
+        "addc.cc.u32 %2, %10, %18;\n\t"
+        "addc.cc.u32 %3, %11, %19;\n\t"
+        "addc.cc.u32 %4, %12, %20;\n\t"
+        "addc.cc.u32 %5, %13, %21;\n\t"
+        "addc.cc.u32 %6, %14, %22;\n\t"
+        "addc.u32    %7, %15, %23;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7])
+        : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]),
+          "r"(D::D0 & mask), "r"(D::D1 & mask), "r"(D::D2 & mask), "r"(D::D3 & mask),
+          "r"(D::D4 & mask), "r"(D::D5 & mask), "r"(D::D6 & mask), "r"(D::D7 & mask));
+}
+
+// r congruent to a - b for loose a, b, only to be multiplied by a factor: where
+// 4p < 2^256, a + 2p - b in (0, 4p) without a correction
+template <class F>
+__device__ __forceinline__ void diff_loose(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
+    using D = Twice<F>;
+    if constexpr (!D::SUM_FITS) {
+        sub_loose<F>(r, a, b);
+    } else {
+        uint32_t u[8];
+        asm("add.cc.u32  %0, %8, %16;\n\t"
+            "addc.cc.u32 %1, %9, %17;\n\t"
+            "addc.cc.u32 %2, %10, %18;\n\t"
+            "addc.cc.u32 %3, %11, %19;\n\t"
+            "addc.cc.u32 %4, %12, %20;\n\t"
+            "addc.cc.u32 %5, %13, %21;\n\t"
+            "addc.cc.u32 %6, %14, %22;\n\t"
+            "addc.u32    %7, %15, %23;"
+            : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
+              "=r"(u[7])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
+              "n"(D::D0), "n"(D::D1), "n"(D::D2), "n"(D::D3), "n"(D::D4), "n"(D::D5), "n"(D::D6),
+              "n"(D::D7));
+        asm("sub.cc.u32  %0, %8, %16;\n\t"
+            "subc.cc.u32 %1, %9, %17;\n\t"
+            "subc.cc.u32 %2, %10, %18;\n\t"
+            "subc.cc.u32 %3, %11, %19;\n\t"
+            "subc.cc.u32 %4, %12, %20;\n\t"
+            "subc.cc.u32 %5, %13, %21;\n\t"
+            "subc.cc.u32 %6, %14, %22;\n\t"
+            "subc.u32    %7, %15, %23;"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+              "=r"(r[7])
+            : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]),
+              "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]),
+              "r"(b[7]));
+    }
+}
+
 // r = a + p - b, in (0, 2p) and congruent to a - b, for canonical a, b: no
 // conditional correction.  Only for values that feed mul as its second
 // (limb-scanned) operand, which may be any value below 2^256.
@@ -357,10 +495,10 @@ __device__ __forceinline__ void mul(uint32_t r[8], const uint32_t a[8], const ui
 //     t  = low 256 bits of x w + q (2^256 - r)
 // Bounds: w' loses less than 1, so x w'/2^256 loses less than x/2^256 < 1; the
 // dropped columns 0..5 are below 7 * 2^224, so they cost q less than 2^-29; the
-// floor costs less than 1.  Hence 0 <= x w - q r < (x/2^256 + 1 + 2^-29) r, below 2r for
-// every x <= 2^256 - 2^228, in particular for x in [0, 2r) (2r < 2^256 - 2^251
-// for the three fields); one conditional subtraction makes it canonical.  If x
-// is a value in Montgomery form, so is the result: w itself is not in it.
+// floor costs less than 1.  Hence 0 <= x w - q r < (x/2^256 + 1 + 2^-29) r, below
+// 2r for every x <= 2^256 - 2^228, in particular for loose x and differences
+// of them (2r, and where it is below 2^256 4r, stay under 2^256 - 2^251).  If x is
+// a value in Montgomery form, so is the result: w itself is not in it.
 //
 // Work on the heavy FMA datapath: 43 + 28 wide multiply-adds and 8 low ones for
 // q and x w, and 15 and 6 (BLS12-381: r_0 = 1, r_1 = 2^32 - 1 leave two limbs of
@@ -374,7 +512,7 @@ __device__ __forceinline__ void mul(uint32_t r[8], const uint32_t a[8], const ui
 // of columns of even and odd index, a wide multiply-add's two words side by
 // side, so that each pair becomes one instruction (see the Montgomery product).
 // ZK_MUL starts a pair of words, ZK_MAD heads a carry chain, ZK_MADC continues
-// it; a trailing H: the high word is new (no addend), LH: both are, L: only the
+// it; a trailing LH: the pair is new, its addend only the carry in; L: only the
 // low word of the product, into the last column.  ZK_CARRY stores a carry out.
 #define ZK_MUL(l, h, a, b) "mul.wide.u32 t, " #a ", " #b ";\n\tmov.b64 {" #l ", " #h "}, t;\n\t"
 #define ZK_MAD2_(c, l, h, a, b, x, y)                                     \
@@ -382,39 +520,45 @@ __device__ __forceinline__ void mul(uint32_t r[8], const uint32_t a[8], const ui
     "madc.hi.cc.u32 " #h ", " #a ", " #b ", " y ";\n\t"
 #define ZK_MAD(l, h, a, b) ZK_MAD2_("", l, h, a, b, #l, #h)
 #define ZK_MADC(l, h, a, b) ZK_MAD2_("c", l, h, a, b, #l, #h)
-#define ZK_MADCH(l, h, a, b) ZK_MAD2_("c", l, h, a, b, #l, "0")
 #define ZK_MADCLH(l, h, a, b) ZK_MAD2_("c", l, h, a, b, "0", "0")
 #define ZK_MULL(l, a, b) "mul.lo.u32 " #l ", " #a ", " #b ";\n\t"
 #define ZK_MADL(l, a, b) "mad.lo.u32 " #l ", " #a ", " #b ", " #l ";\n\t"
-#define ZK_MADCL(l, a, b) "madc.lo.u32 " #l ", " #a ", " #b ", " #l ";\n\t"
+// (the carry by an add of its own: a narrow multiply-add with carry in holds the
+// heavy datapath for four cycles, without it for two)
+#define ZK_MADCL(l, a, b) "addc.u32 " #l ", " #l ", 0;\n\t" ZK_MADL(l, a, b)
 #define ZK_CARRY(l) "addc.u32 " #l ", 0, 0;\n\t"
 #define ZK_NAME8(n, a, b, c, d, e, f, g, h)                                              \
     ".reg .u32 " #n "<8>;\n\t"                                                           \
     "mov.u32 " #n "0, " a "; mov.u32 " #n "1, " b "; mov.u32 " #n "2, " c "; mov.u32 " #n "3, " d ";\n\t" \
     "mov.u32 " #n "4, " e "; mov.u32 " #n "5, " f "; mov.u32 " #n "6, " g "; mov.u32 " #n "7, " h ";\n\t"
 
-// columns 6..14 of x y
-#define ZK_ROWS_HIGH                                                                               \
-    ZK_MUL(e6, e7, x0, y6) ZK_MUL(o7, o8, x0, y7)                                                  \
-    ZK_MAD(e6, e7, x1, y5) ZK_MADCLH(e8, e9, x1, y7) ZK_MAD(o7, o8, x1, y6) ZK_CARRY(o9)           \
-    ZK_MAD(e6, e7, x2, y4) ZK_MADC(e8, e9, x2, y6) ZK_CARRY(e10) ZK_MAD(o7, o8, x2, y5)            \
-    ZK_MADCH(o9, o10, x2, y7)                                                                      \
-    ZK_MAD(e6, e7, x3, y3) ZK_MADC(e8, e9, x3, y5) ZK_MADCH(e10, e11, x3, y7)                      \
-    ZK_MAD(o7, o8, x3, y4) ZK_MADC(o9, o10, x3, y6) ZK_CARRY(o11)                                  \
-    ZK_MAD(e6, e7, x4, y2) ZK_MADC(e8, e9, x4, y4) ZK_MADC(e10, e11, x4, y6) ZK_CARRY(e12)         \
-    ZK_MAD(o7, o8, x4, y3) ZK_MADC(o9, o10, x4, y5) ZK_MADCH(o11, o12, x4, y7)                     \
-    ZK_MAD(e6, e7, x5, y1) ZK_MADC(e8, e9, x5, y3) ZK_MADC(e10, e11, x5, y5)                       \
-    ZK_MADCH(e12, e13, x5, y7) ZK_MAD(o7, o8, x5, y2) ZK_MADC(o9, o10, x5, y4)                     \
-    ZK_MADC(o11, o12, x5, y6) ZK_CARRY(o13)                                                        \
-    ZK_MAD(e6, e7, x6, y0) ZK_MADC(e8, e9, x6, y2) ZK_MADC(e10, e11, x6, y4)                       \
-    ZK_MADC(e12, e13, x6, y6) ZK_CARRY(e14) ZK_MAD(o7, o8, x6, y1) ZK_MADC(o9, o10, x6, y3)        \
-    ZK_MADC(o11, o12, x6, y5) ZK_MADCH(o13, o14, x6, y7)                                           \
-    ZK_MAD(e8, e9, x7, y1) ZK_MADC(e10, e11, x7, y3) ZK_MADC(e12, e13, x7, y5)                     \
-    ZK_MADCH(e14, e15, x7, y7) ZK_MAD(o7, o8, x7, y0) ZK_MADC(o9, o10, x7, y2)                     \
-    ZK_MADC(o11, o12, x7, y4) ZK_MADC(o13, o14, x7, y6) ZK_CARRY(o15)
-// columns 0..7 of x w
+// columns 6..14 of x y.  A row's carries out are single bits.  That of the odd
+// columns is kept as the low word of the next row's top pair; that of the even
+// columns (rows 2, 4, 6) as the high word of the same row's odd top pair, which
+// is otherwise new: x_i y_7 < 2^64 - 2^33 + 2 leaves room for both.
+#define ZK_ROWS_HIGH                                                                                   \
+    ZK_MUL(e6, e7, x0, y6) ZK_MUL(o7, o8, x0, y7)                                                      \
+    ZK_MAD(e6, e7, x1, y5) ZK_MADCLH(e8, e9, x1, y7) ZK_MAD(o7, o8, x1, y6) ZK_CARRY(o9)               \
+    ZK_MAD(e6, e7, x2, y4) ZK_MADC(e8, e9, x2, y6) ZK_CARRY(o10)                                       \
+    ZK_MAD(o7, o8, x2, y5) ZK_MADC(o9, o10, x2, y7)                                                    \
+    ZK_MAD(e6, e7, x3, y3) ZK_MADC(e8, e9, x3, y5) ZK_MADCLH(e10, e11, x3, y7)                         \
+    ZK_MAD(o7, o8, x3, y4) ZK_MADC(o9, o10, x3, y6) ZK_CARRY(o11)                                      \
+    ZK_MAD(e6, e7, x4, y2) ZK_MADC(e8, e9, x4, y4) ZK_MADC(e10, e11, x4, y6) ZK_CARRY(o12)             \
+    ZK_MAD(o7, o8, x4, y3) ZK_MADC(o9, o10, x4, y5) ZK_MADC(o11, o12, x4, y7)                          \
+    ZK_MAD(e6, e7, x5, y1) ZK_MADC(e8, e9, x5, y3) ZK_MADC(e10, e11, x5, y5) ZK_MADCLH(e12, e13, x5, y7)\
+    ZK_MAD(o7, o8, x5, y2) ZK_MADC(o9, o10, x5, y4) ZK_MADC(o11, o12, x5, y6) ZK_CARRY(o13)            \
+    ZK_MAD(e6, e7, x6, y0) ZK_MADC(e8, e9, x6, y2) ZK_MADC(e10, e11, x6, y4) ZK_MADC(e12, e13, x6, y6) \
+    ZK_CARRY(o14) ZK_MAD(o7, o8, x6, y1) ZK_MADC(o9, o10, x6, y3) ZK_MADC(o11, o12, x6, y5)            \
+    ZK_MADC(o13, o14, x6, y7)                                                                          \
+    ZK_MAD(e8, e9, x7, y1) ZK_MADC(e10, e11, x7, y3) ZK_MADC(e12, e13, x7, y5) ZK_MADCLH(e14, e15, x7, y7)\
+    ZK_MAD(o7, o8, x7, y0) ZK_MADC(o9, o10, x7, y2) ZK_MADC(o11, o12, x7, y4) ZK_MADC(o13, o14, x7, y6)\
+    ZK_CARRY(o15)
+// columns 0..7 of x w: the first row's even columns, new or added to e, and the rest
+#define ZK_ROW_LOW_NEW                                                                              \
+    ZK_MUL(e0, e1, x0, w0) ZK_MUL(e2, e3, x0, w2) ZK_MUL(e4, e5, x0, w4) ZK_MUL(e6, e7, x0, w6)
+#define ZK_ROW_LOW_ADD                                                                              \
+    ZK_MAD(e0, e1, x0, w0) ZK_MADC(e2, e3, x0, w2) ZK_MADC(e4, e5, x0, w4) ZK_MADC(e6, e7, x0, w6)
 #define ZK_ROWS_LOW                                                                                \
-    ZK_MUL(e0, e1, x0, w0) ZK_MUL(e2, e3, x0, w2) ZK_MUL(e4, e5, x0, w4) ZK_MUL(e6, e7, x0, w6)    \
     ZK_MUL(o1, o2, x0, w1) ZK_MUL(o3, o4, x0, w3) ZK_MUL(o5, o6, x0, w5) ZK_MULL(o7, x0, w7)       \
     ZK_MAD(e2, e3, x1, w1) ZK_MADC(e4, e5, x1, w3) ZK_MADC(e6, e7, x1, w5)                         \
     ZK_MAD(o1, o2, x1, w0) ZK_MADC(o3, o4, x1, w2) ZK_MADC(o5, o6, x1, w4) ZK_MADCL(o7, x1, w6)    \
@@ -494,11 +638,11 @@ __device__ __forceinline__ void mul_low_fold(uint32_t t[8], const uint32_t x[8],
     ZK_NAME8(w, "%16", "%17", "%18", "%19", "%20", "%21", "%22", "%23")            \
     ZK_NAME8(q, "%24", "%25", "%26", "%27", "%28", "%29", "%30", "%31")            \
     ZK_NAME8(n, "%32", "%33", "%34", "%35", "%36", "%37", "%38", "%39")
-#define ZK_LOW_SUB_Q  /* q (2^32 - 1): minus q, and plus q one limb up in n_1 */   \
-    "sub.cc.u32 e0, e0, q0;\n\tsubc.cc.u32 e1, e1, q1;\n\t"                      \
-    "subc.cc.u32 e2, e2, q2;\n\tsubc.cc.u32 e3, e3, q3;\n\t"                     \
-    "subc.cc.u32 e4, e4, q4;\n\tsubc.cc.u32 e5, e5, q5;\n\t"                     \
-    "subc.cc.u32 e6, e6, q6;\n\tsubc.u32 e7, e7, q7;\n\t"
+#define ZK_LOW_Q  /* q (2^32 - 1) = (q << 32) - q */                               \
+    "sub.cc.u32 e0, 0, q0;\n\tsubc.cc.u32 e1, q0, q1;\n\t"                       \
+    "subc.cc.u32 e2, q1, q2;\n\tsubc.cc.u32 e3, q2, q3;\n\t"                     \
+    "subc.cc.u32 e4, q3, q4;\n\tsubc.cc.u32 e5, q4, q5;\n\t"                     \
+    "subc.cc.u32 e6, q5, q6;\n\tsubc.u32 e7, q6, q7;\n\t"
 #define ZK_LOW_TAIL                                                                \
     "mov.u32 %0, e0;\n\t"                                                          \
     "add.cc.u32 %1, e1, o1;\n\taddc.cc.u32 %2, e2, o2;\n\t"                      \
@@ -511,19 +655,17 @@ __device__ __forceinline__ void mul_low_fold(uint32_t t[8], const uint32_t x[8],
       "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7]),                \
       "n"(n0), "n"(n1), "n"(~F::P2), "n"(~F::P3), "n"(~F::P4), "n"(~F::P5), "n"(~F::P6), "n"(~F::P7)
     if constexpr (F::P0 == 1u && F::P1 == 0xffffffffu) {
-        asm(ZK_LOW_HEAD ZK_ROWS_LOW ZK_ROWS_N2 ZK_LOW_SUB_Q
-            "add.cc.u32 e1, e1, q0;\n\taddc.cc.u32 e2, e2, q1;\n\t"
-            "addc.cc.u32 e3, e3, q2;\n\taddc.cc.u32 e4, e4, q3;\n\t"
-            "addc.cc.u32 e5, e5, q4;\n\taddc.cc.u32 e6, e6, q5;\n\taddc.u32 e7, e7, q6;\n\t"
-            ZK_LOW_TAIL ZK_LOW_OPERANDS(0, 0));
+        asm(ZK_LOW_HEAD ZK_LOW_Q ZK_ROW_LOW_ADD ZK_ROWS_LOW ZK_ROWS_N2 ZK_LOW_TAIL
+            ZK_LOW_OPERANDS(0, 0));
     } else if constexpr (F::P0 == 1u) {
-        asm(ZK_LOW_HEAD ZK_ROWS_LOW ZK_ROWS_N1 ZK_LOW_SUB_Q ZK_LOW_TAIL
-            ZK_LOW_OPERANDS(0, 0u - F::P1));
+        asm(ZK_LOW_HEAD ZK_LOW_Q ZK_ROW_LOW_ADD ZK_ROWS_LOW ZK_ROWS_N1 ZK_LOW_TAIL
+            ZK_LOW_OPERANDS(0, ~F::P1));
     } else {
-        asm(ZK_LOW_HEAD ZK_ROWS_LOW ZK_ROWS_N0 ZK_LOW_TAIL ZK_LOW_OPERANDS(0u - F::P0, ~F::P1));
+        asm(ZK_LOW_HEAD ZK_ROW_LOW_NEW ZK_ROWS_LOW ZK_ROWS_N0 ZK_LOW_TAIL
+            ZK_LOW_OPERANDS(0u - F::P0, ~F::P1));
     }
 #undef ZK_LOW_HEAD
-#undef ZK_LOW_SUB_Q
+#undef ZK_LOW_Q
 #undef ZK_LOW_TAIL
 #undef ZK_LOW_OPERANDS
 }
@@ -534,13 +676,12 @@ struct Factor {
     uint32_t w[8], wq[8];
 };
 
-// r = x f mod p, canonical, for any x <= 2^256 - 2^228 (x in [0, 2p) is)
+// r = x f mod p, loose (in [0, 2p)), for any x <= 2^256 - 2^228
 template <class F>
 __device__ __forceinline__ void mul_factor(uint32_t r[8], const uint32_t x[8], const Factor &f) {
     uint32_t q[8], t[8];
     mul_high(q, x, f.wq);
     mul_low_fold<F>(t, x, f.w, q);
-    reduce_once<F>(t);
 #pragma unroll
     for (int i = 0; i < 8; i++) r[i] = t[i];
 }
@@ -550,7 +691,7 @@ __device__ __forceinline__ void mul_low(uint32_t t[8], const uint32_t x[8], cons
     asm("{\n\t.reg .u32 e<16>, o<16>;\n\t.reg .u64 t;\n\t"
         ZK_NAME8(x, "%8", "%9", "%10", "%11", "%12", "%13", "%14", "%15")
         ZK_NAME8(w, "%16", "%17", "%18", "%19", "%20", "%21", "%22", "%23")
-        ZK_ROWS_LOW
+        ZK_ROW_LOW_NEW ZK_ROWS_LOW
         "mov.u32 %0, e0;\n\t"
         "add.cc.u32 %1, e1, o1;\n\taddc.cc.u32 %2, e2, o2;\n\t"
         "addc.cc.u32 %3, e3, o3;\n\taddc.cc.u32 %4, e4, o4;\n\t"
@@ -614,6 +755,13 @@ __device__ __forceinline__ void ld_elem_cg(uint32_t x[8], const uint4 *p) {
 __device__ __forceinline__ void st_elem(uint4 *p, const uint32_t x[8]) {
     p[0] = make_uint4(x[0], x[1], x[2], x[3]);
     p[1] = make_uint4(x[4], x[5], x[6], x[7]);
+}
+
+// one 32-byte store a lane: a whole sector in one request
+__device__ __forceinline__ void st_elem8(uint4 *p, const uint32_t x[8]) {
+    asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(x[0]), "r"(x[1]),
+                 "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7]), "l"(p)
+                 : "memory");
 }
 
 __device__ __forceinline__ void st_factor(uint4 *p, const Factor &f) {

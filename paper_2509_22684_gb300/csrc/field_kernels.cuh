@@ -1,0 +1,54 @@
+// field_kernels.cuh -- the kernel table of one field (included by the
+// field-specific translation units).
+#pragma once
+#include "aux_kernels.cuh"
+#include "kernels.h"
+#include "ntt_pass.cuh"
+
+namespace zkntt {
+
+// the pass kernels compiled for a digit of K bits: one thread per four elements
+// of a tile, 96 registers (128 when that makes 256 threads)
+template <class F, int K, Kind KIND>
+const void *fixed_kernel() {
+    constexpr int T = 1 << (K + fixed_cols(K) - 2);
+    constexpr int B = T >= 256 ? 2 : T >= 32 ? 640 / T : 20;
+    return (const void *)&ntt_pass_kernel<F, T, B, RADIX4, K, KIND>;
+}
+
+template <class F, int K>
+void set_fixed(FieldKernels &k) {
+    k.fixed[K][STRIDED] = fixed_kernel<F, K, STRIDED>();
+    k.fixed[K][STRIDED_PRE] = fixed_kernel<F, K, STRIDED_PRE>();
+    k.fixed[K][STRIDED_OTF] = fixed_kernel<F, K, STRIDED_OTF>();
+    k.fixed[K][LAST] = fixed_kernel<F, K, LAST>();
+    k.fixed[K][LAST_POST] = fixed_kernel<F, K, LAST_POST>();
+}
+
+template <class F>
+FieldKernels make_field_kernels() {
+    FieldKernels k = {};
+    // registers: 96 (variants 1 and 7), 128 (2 and 4), 80 (3 and 6), 64 (5)
+    k.pass[1] = k.pass[7] = (const void *)&ntt_pass_kernel<F, 128, 5, RADIX4, 0, ANY>;
+    k.pass[2] = k.pass[4] = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX4, 0, ANY>;
+    k.pass[3] = k.pass[6] = (const void *)&ntt_pass_kernel<F, 256, 3, RADIX4, 0, ANY>;
+    k.pass[5] = (const void *)&ntt_pass_kernel<F, 256, 4, RADIX2, 0, ANY>;
+    set_fixed<F, 5>(k);
+    set_fixed<F, 6>(k);
+    set_fixed<F, 7>(k);
+    set_fixed<F, 8>(k);
+    set_fixed<F, 9>(k);
+    set_fixed<F, 10>(k);
+    k.gen_powers = (const void *)&gen_powers_kernel<F>;
+    k.gen_twiddle = (const void *)&gen_twiddle_kernel<F>;
+    k.field_op = (const void *)&field_op_kernel<F>;
+    k.pointwise = (const void *)&pointwise_kernel<F>;
+    k.mulbench = (const void *)&mulbench_kernel<F>;
+    k.scale_powers = (const void *)&scale_powers_kernel<F>;
+    k.block_dft[1] = (const void *)&block_dft_kernel<F, 2>;
+    k.block_dft[2] = (const void *)&block_dft_kernel<F, 4>;
+    k.block_dft[3] = (const void *)&block_dft_kernel<F, 8>;
+    return k;
+}
+
+}  // namespace zkntt

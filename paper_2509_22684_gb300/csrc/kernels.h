@@ -10,6 +10,7 @@ constexpr int MAX_TILE_BITS = 11;   // tiles hold at most 2^11 elements (C x 2^K
 
 struct FieldKernels {
     const void *pass[8];  // the pass kernel of schedule variant 1..7 (digit size is a runtime argument)
+    const void *fixed[MAX_DIGIT_BITS + 1][6];  // pass kernels by digit bits and Kind (null: none)
     const void *gen_powers;
     const void *gen_twiddle;
     const void *field_op;
@@ -27,8 +28,6 @@ const FieldKernels &kernels_bls12_377();
 constexpr int NUM_FIELDS = 3;
 // pass-kernel schedule variants, 1 .. NUM_VARIANTS (the plan's `ilp` option)
 constexpr int NUM_VARIANTS = 7;
-// variants the autotuner tries (1 .. TUNED_VARIANTS)
-constexpr int TUNED_VARIANTS = 5;
 const void *batch_kernel_ptr(int field);
 // the 32-bit multiply-add rate calibration kernel (field-independent)
 const void *imadbench_kernel_ptr();

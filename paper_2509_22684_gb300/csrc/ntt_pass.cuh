@@ -28,12 +28,15 @@
 // All sizes (K, C, the stride) are runtime values: one kernel per field serves
 // every digit size.
 //
-// Shared memory holds each element as two 16-byte halves in separate arrays.
-// The slot of (column c, row d) is c*N + (d ^ s), with s in the low three bits
-// a linear function of bits 3 and 4 of d and of c (smem_slot), chosen so that
-// the eight lanes of an access fall into different bank groups in every
-// pattern: copies with columns or rows fastest, steps at distance 4 and above,
-// and the last step on rows 4 g + i with columns fastest.
+// Values are residues in [0, 2r) throughout; the last pass brings its outputs
+// below r.
+//
+// Shared memory holds elements in groups of eight: eight low 16-byte halves,
+// then the eight high ones.  The slot of (column c, row d) is c*N + (d ^ s), with
+// s in the low three bits a linear function of bits 3 and 4 of d and of c
+// (smem_unit), chosen so that the eight lanes of an access fall into different
+// bank groups in every pattern: copies with columns or rows fastest, steps at
+// distance 4 and above, and the last step on rows 4 g + i with columns fastest.
 //
 // Per-element factors (one product each, only when present), all held as
 // (w, quotient) pairs of 64 bytes for mul_factor:
@@ -79,18 +82,34 @@ __device__ __forceinline__ uint32_t brev_bits(uint32_t x, uint32_t bits) {
     return bits == 0 ? 0u : (__brev(x) >> (32 - bits));
 }
 
-// Row part of the shared-memory slot (K >= 3): d with its low three bits
-// xor 5 for bit 3 and xor 6 for bit 4.  Linear over xor, so the rows of a group
-// at distances that are powers of two have slots at xor distances.
-__device__ __forceinline__ uint32_t row_slot(uint32_t d) {
-    return d ^ (((d >> 3) & 1u) * 5u) ^ (((d >> 4) & 1u) * 6u);
+// Place of slot s among the 16-byte units of shared memory: the low half, and
+// the high one HALF units on.
+constexpr uint32_t HALF = 8;
+__host__ __device__ __forceinline__ uint32_t slot_unit(uint32_t s) {
+    return ((s & ~7u) << 1) | (s & 7u);
 }
 
-// shared-memory slot of element (column c, row d)
-__device__ __forceinline__ uint32_t smem_slot(uint32_t c, uint32_t d, uint32_t K, uint32_t lc) {
-    if (K < 3) return (c << K) + d;
+// units of a tile of CN elements
+__host__ __device__ constexpr uint32_t tile_units(uint32_t CN) { return CN < 8 ? 16u : 2 * CN; }
+
+// Row part of an element's unit (K >= 3): d with its low three bits xor 5 for
+// bit 3 and xor 6 for bit 4 (0, 5, 6, 3 by the two bits).  Linear over xor, so
+// the rows of a group at distances that are powers of two have units at xor
+// distances.
+__device__ __forceinline__ uint32_t row_unit(uint32_t d) {
+    return slot_unit(d ^ ((0x3650u >> ((d >> 1) & 12u)) & 7u));
+}
+
+// column part of an element's unit, to be xor-ed to the row's
+__device__ __forceinline__ uint32_t col_unit(uint32_t c, uint32_t K, uint32_t lc) {
+    if (K < 3) return slot_unit(c << K);
     const uint32_t s = lc == 3 ? c : lc == 2 ? ((c & 1u) << 1) ^ ((c >> 1) * 5u) : c * 6u;
-    return (c << K) + (row_slot(d) ^ s);
+    return (c << (K + 1)) | s;
+}
+
+// unit of element (column c, row d)
+__device__ __forceinline__ uint32_t smem_unit(uint32_t c, uint32_t d, uint32_t K, uint32_t lc) {
+    return K < 3 ? slot_unit((c << K) + d) : col_unit(c, K, lc) ^ row_unit(d);
 }
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
@@ -107,17 +126,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
-__device__ __forceinline__ void lds_elem(uint32_t x[8], const uint4 *s_lo, const uint4 *s_hi,
-                                         uint32_t slot) {
-    uint4 v0 = s_lo[slot], v1 = s_hi[slot];
+__device__ __forceinline__ void lds_elem(uint32_t x[8], const uint4 *buf, uint32_t unit) {
+    const uint4 v0 = buf[unit], v1 = buf[unit + HALF];
     x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w;
     x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
 }
 
-__device__ __forceinline__ void sts_elem(uint4 *s_lo, uint4 *s_hi, uint32_t slot,
-                                         const uint32_t x[8]) {
-    s_lo[slot] = make_uint4(x[0], x[1], x[2], x[3]);
-    s_hi[slot] = make_uint4(x[4], x[5], x[6], x[7]);
+__device__ __forceinline__ void sts_elem(uint4 *buf, uint32_t unit, const uint32_t x[8]) {
+    buf[unit] = make_uint4(x[0], x[1], x[2], x[3]);
+    buf[unit + HALF] = make_uint4(x[4], x[5], x[6], x[7]);
 }
 
 // Global index of tile element (row d, column cc) before (src) and after (dst)
@@ -134,118 +151,174 @@ __device__ __forceinline__ size_t tile_src(const PassArgs &a, uint32_t tile, uin
     return (size_t(brev_bits(b, a.hi_bits)) << a.K) + d;
 }
 
-__device__ __forceinline__ size_t tile_dst(const PassArgs &a, uint32_t tile, uint32_t d,
-                                           uint32_t cc) {
-    if (!a.last) return tile_src(a, tile, d, cc);
-    return (size_t(brev_bits(d, a.K)) << a.hi_bits) + (size_t(tile) << a.log_cols) + cc;
-}
-
-// The factors of row position d in column cc on the way out: the inter-pass
-// twiddle (precomputed, or up to four factors on the fly) or the last pass's
-// post scale.  A null p[0]: none; a null p[k] ends the list.
-__device__ __forceinline__ void out_factors(const uint4 *p[4], const PassArgs &a, uint32_t tile,
+// The factors of row position d in column cc on the way out, formed on the fly:
+// a null p[k] ends the list.
+__device__ __forceinline__ void otf_factors(const uint4 *p[4], const PassArgs &a, uint32_t tile,
                                             uint32_t d, uint32_t cc) {
-    p[0] = p[1] = p[2] = p[3] = nullptr;
-    if (a.last) {
-        if (a.post) p[0] = a.post + 4 * size_t(d);
-        return;
-    }
     const uint32_t lo_tiles_bits = a.lo_bits - a.log_cols;
     const uint32_t lo = ((tile & ((1u << lo_tiles_bits) - 1u)) << a.log_cols) + cc;
-    if (!a.otf) {
-        p[0] = a.tw + 4 * ((size_t(d) << a.lo_bits) + lo);
-        return;
-    }
     // lo < 2^lo_bits and rev(d) < 2^K, so e < 2^tw_bits = n_i: no reduction
     // (and no overflow: tw_bits <= 32)
     const uint32_t e = lo * brev_bits(d, a.K);
     p[0] = a.w_hi + 4 * size_t(e >> a.split_bits);
     p[1] = a.w_lo + 4 * size_t(e & ((1u << a.split_bits) - 1u));
+    p[2] = p[3] = nullptr;
     if (a.fl) p[2] = a.fl + 4 * size_t(lo);
     if (a.fd) (a.fl ? p[3] : p[2]) = a.fd + 4 * size_t(d);
 }
 
-// x times its output factors, to its place in global memory.  One product in
-// the code, in a loop over the factors: unrolled, the kernels outgrow the
-// instruction cache.
-template <class F>
-__device__ __forceinline__ void scale_and_store(uint32_t x[8], const PassArgs &a, uint32_t tile,
-                                                uint32_t d, uint32_t cc) {
-    const uint4 *p[4];
-    out_factors(p, a, tile, d, cc);
-    // an entry of the big table is read once: it takes no place in L1
-    const bool stream = !a.last && !a.otf;
-#pragma unroll 1
-    while (p[0]) {
-        Factor f;
-        if (stream) ldg_factor_stream(f, p[0]);
-        else ldg_factor(f, p[0]);
-        mul_factor<F>(x, x, f);
-        p[0] = p[1];
-        p[1] = p[2];
-        p[2] = p[3];
-        p[3] = nullptr;
+// Where a thread's rows d0 .. d0 + R - 1 of column cc go (R = 4, or 2 when
+// N = 2; d0 a multiple of R), and their factors: row d0 + i, in order of i in a
+// strided pass, of rev(i) in the last, is `step` elements on from the one before;
+// its factor (null: none, or on the fly) is `fstep` units on in order of i.
+struct OutRows {
+    uint4 *out;
+    size_t step, fstep;
+    const uint4 *f;
+};
+template <int R>
+__device__ __forceinline__ OutRows out_rows(const PassArgs &a, uint32_t tile, uint32_t d0,
+                                            uint32_t cc) {
+    OutRows o;
+    if (a.last) {
+        o.out = a.out + 2 * ((size_t(brev_bits(d0, a.K)) << a.hi_bits) +
+                             (size_t(tile) << a.log_cols) + cc);
+        o.step = size_t(1) << (a.K - (R == 4 ? 2 : 1) + a.hi_bits);
+        o.f = a.post ? a.post + 4 * size_t(d0) : nullptr;
+        o.fstep = 4;
+    } else {
+        const uint32_t lo_tiles_bits = a.lo_bits - a.log_cols;
+        const uint32_t lo = ((tile & ((1u << lo_tiles_bits) - 1u)) << a.log_cols) + cc;
+        const size_t hi = tile >> lo_tiles_bits;
+        o.out = a.out + 2 * (((hi << a.K | d0) << a.lo_bits) + lo);
+        o.step = size_t(1) << a.lo_bits;
+        o.f = a.otf ? nullptr : a.tw + 4 * ((size_t(d0) << a.lo_bits) + lo);
+        o.fstep = 4 * o.step;
     }
-    st_elem(a.out + 2 * tile_dst(a, tile, d, cc), x);
+    return o;
+}
+
+// The rows at units u0 ^ i, times their output factors, to global memory: a
+// loop with one product in the code (unrolled, the kernels outgrow the
+// instruction cache).  The table's factor of the next row is read into the
+// registers of the present one as soon as the product is done with them: its
+// quotient during the second half of the product, its value during the store and
+// the first half of the next.
+template <class F, int R>
+__device__ __forceinline__ void scale_and_store(const PassArgs &a, const uint4 *buf, uint32_t u0,
+                                                const OutRows &o, uint32_t tile, uint32_t d0,
+                                                uint32_t cc) {
+    if (o.f) {
+        Factor v;
+        // (an entry of the big table is read once: it takes no place in L1)
+        if (a.last) ldg_factor(v, o.f);
+        else ldg_factor_stream(v, o.f);
+        const uint4 *f = o.f;
+#pragma unroll 1
+        for (uint32_t i = 0; i < R; i++) {
+            uint32_t x[8], q[8];
+            lds_elem(x, buf, u0 ^ i);
+            mul_high(q, x, v.wq);
+            if (i + 1 < R) f += o.fstep;
+            if (a.last) ZK_LD8("", v.wq, f + 2);
+            else ZK_LD8(".L1::no_allocate", v.wq, f + 2);
+            mul_low_fold<F>(x, x, v.w, q);
+            if (a.last) ZK_LD8("", v.w, f);
+            else ZK_LD8(".L1::no_allocate", v.w, f);
+            uint32_t r = i;
+            if (a.last) {
+                reduce_once<F>(x);
+                if (R == 4) r = ((i & 1u) << 1) | (i >> 1);
+            }
+            st_elem8(o.out + 2 * r * o.step, x);
+        }
+        return;
+    }
+#pragma unroll 1
+    for (uint32_t i = 0; i < R; i++) {
+        const uint4 *p[4];
+        otf_factors(p, a, tile, d0 + i, cc);
+        uint32_t x[8];
+        lds_elem(x, buf, u0 ^ i);
+#pragma unroll 1
+        while (p[0]) {
+            Factor v;
+            ldg_factor(v, p[0]);
+            mul_factor<F>(x, x, v);
+            p[0] = p[1];
+            p[1] = p[2];
+            p[2] = p[3];
+            p[3] = nullptr;
+        }
+        st_elem8(o.out + 2 * i * o.step, x);
+    }
 }
 
 // Issue (without waiting) the 16-byte copies of one tile into shared memory:
 // 8 lanes copy the low halves of 8 elements, the next 8 lanes their high
 // halves (tiles under 8 elements: element-major); columns fastest for strided
 // passes, rows fastest for the last.
-__device__ __forceinline__ void issue_tile_load(const PassArgs &a, uint4 *smem, uint32_t tile,
+__device__ __forceinline__ void issue_tile_load(const PassArgs &a, uint4 *buf, uint32_t tile,
                                                 uint32_t nthreads) {
     const uint32_t K = a.K, lc = a.log_cols;
     const uint32_t N = 1u << K, C = 1u << lc, CN = C << K;
-    uint4 *s_lo = smem, *s_hi = smem + CN;
     const uint32_t tid = threadIdx.x;
     if (tid >= nthreads) return;
     if (CN >= 64 && (nthreads & 15u) == 0 && (nthreads & (nthreads - 1u)) == 0 && nthreads <= 2 * CN) {
         // Every thread makes 2 C N / nthreads copies of one half (the lane's
-        // bit 3) of elements e0, e0 + E, e0 + 2E, ... (E = nthreads / 2); in
-        // a strided pass they share a column and step by a fixed row count,
-        // so the source address steps by a fixed stride and only the shared
-        // slot is formed per copy.
+        // bit 3) of elements e0, e0 + E, e0 + 2E, ... (E = nthreads / 2): rows
+        // at a power-of-two step in one column, so the source steps by a fixed
+        // stride and the units lie at xor distances (the same for all threads).
         const uint32_t half = (tid >> 3) & 1u;
         const uint32_t e0 = (tid & 7u) | ((tid >> 4) << 3);
+        // (four copies at a time: one per four elements makes eight or more)
         const uint32_t E = nthreads >> 1, iters = (2 * CN) / nthreads;
-        const uint32_t sbase =
-            static_cast<uint32_t>(__cvta_generic_to_shared(half ? s_hi : s_lo));
-        if (!a.last) {
-            const uint32_t cc = e0 & (C - 1), dstep = E >> lc;
-            uint32_t d = e0 >> lc;
+        const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(buf + half * HALF));
+        if (!a.last && iters >= 4) {
+            const uint32_t cc = e0 & (C - 1), dstep = E >> lc, d = e0 >> lc;
             const uint4 *src = a.in + 2 * tile_src(a, tile, d, cc) + half;
             const size_t sstep = size_t(2 * dstep) << a.lo_bits;
-            if ((dstep & 31u) == 0) {
-                // rows d, d + dstep, ... agree in their low five bits, so they
-                // share the swizzle term and their slots step by dstep too
-                uint32_t sa = sbase + 16u * smem_slot(cc, d, K, lc);
-                for (uint32_t k = 0; k < iters; k++, sa += 16u * dstep, src += sstep)
-                    cp_async16_sa(sa, src);
-            } else {
-                for (uint32_t k = 0; k < iters; k++, d += dstep, src += sstep)
-                    cp_async16_sa(sbase + 16u * smem_slot(cc, d, K, lc), src);
+            const uint32_t u1 = row_unit(dstep), u2 = row_unit(2 * dstep);
+            const uint32_t u = smem_unit(cc, d, K, lc);
+#pragma unroll 1
+            for (uint32_t k = 0; k < iters; k += 4, src += 4 * sstep) {
+                const uint32_t v = u ^ row_unit(k * dstep);
+                cp_async16_sa(sbase + 16u * v, src);
+                cp_async16_sa(sbase + 16u * (v ^ u1), src + sstep);
+                cp_async16_sa(sbase + 16u * (v ^ u2), src + 2 * sstep);
+                cp_async16_sa(sbase + 16u * (v ^ u1 ^ u2), src + 3 * sstep);
             }
-        } else if (E < N) {
+        } else if (a.last && 4 * E <= N) {
             // last pass, rows fastest: N / E copies in one column (rows e0,
             // e0 + E, ...; e0 < E), then the next column
             const uint32_t per = N / E;
+            const uint32_t u1 = row_unit(E), u2 = row_unit(2 * E);
+#pragma unroll 1
             for (uint32_t cc = 0; cc < C; cc++) {
-                const uint4 *row = a.in + 2 * tile_src(a, tile, 0, cc) + half;
-                for (uint32_t j = 0, d = e0; j < per; j++, d += E)
-                    cp_async16_sa(sbase + 16u * smem_slot(cc, d, K, lc), row + 2 * d);
+                const uint4 *src = a.in + 2 * tile_src(a, tile, e0, cc) + half;
+                const uint32_t u = smem_unit(cc, e0, K, lc);
+#pragma unroll 1
+                for (uint32_t j = 0; j < per; j += 4, src += 8 * E) {
+                    const uint32_t v = u ^ row_unit(j * E);
+                    cp_async16_sa(sbase + 16u * v, src);
+                    cp_async16_sa(sbase + 16u * (v ^ u1), src + 2 * E);
+                    cp_async16_sa(sbase + 16u * (v ^ u2), src + 4 * E);
+                    cp_async16_sa(sbase + 16u * (v ^ u1 ^ u2), src + 6 * E);
+                }
             }
         } else {
             uint32_t e = e0;
+#pragma unroll 1
             for (uint32_t k = 0; k < iters; k++, e += E) {
                 const uint32_t d = e & (N - 1), cc = e >> K;
-                cp_async16_sa(sbase + 16u * smem_slot(cc, d, K, lc),
+                cp_async16_sa(sbase + 16u * smem_unit(cc, d, K, lc),
                               a.in + 2 * tile_src(a, tile, d, cc) + half);
             }
         }
         return;
     }
     const bool grouped = CN >= 8;
+#pragma unroll 1
     for (uint32_t u = tid; u < 2 * CN; u += nthreads) {
         const uint32_t e = grouped ? ((u & 7u) | ((u >> 4) << 3)) : (u >> 1);
         const uint32_t half = grouped ? ((u >> 3) & 1u) : (u & 1u);
@@ -253,66 +326,81 @@ __device__ __forceinline__ void issue_tile_load(const PassArgs &a, uint4 *smem, 
         if (a.last) { d = e & (N - 1); cc = e >> K; }
         else        { cc = e & (C - 1); d = e >> lc; }
         const size_t g = tile_src(a, tile, d, cc);
-        cp_async16((half ? s_hi : s_lo) + smem_slot(cc, d, K, lc), a.in + 2 * g + half);
+        cp_async16(buf + smem_unit(cc, d, K, lc) + half * HALF, a.in + 2 * g + half);
     }
 }
 
-// The sub-transform's twiddles in shared memory: the N/2 factors w_N^e in four
-// planes of N/2 16-byte quarters, entry e at slot tab_slot(e).  The slot's low
-// three bits fold in the higher ones, so eight entries at any power-of-two
-// stride lie in different bank groups.  (Read from global memory instead, they
-// missed L1 half the time and were two thirds of the load/store wavefronts.)
-__host__ __device__ __forceinline__ uint32_t tab_slot(uint32_t e) {
-    return e ^ (((e >> 3) ^ (e >> 6) ^ (e >> 9)) & 7u);
+// The sub-transform's twiddles in shared memory: the N/2 factors w_N^e in groups
+// of eight, each group as four rows of eight 16-byte quarters.  Entry e's slot
+// is e with its low three bits xor its higher ones in threes, so eight entries at
+// any power-of-two stride lie in different bank groups.  (Read from global
+// memory instead, they missed L1 half the time and were two thirds of the
+// load/store wavefronts.)  tab_unit is linear over xor.
+__host__ __device__ __forceinline__ uint32_t tab_unit(uint32_t e) {
+    return ((e & ~7u) << 2) | ((e ^ (e >> 3) ^ (e >> 6) ^ (e >> 9)) & 7u);
 }
 
-// entries of the table of a 2^K-point sub-transform
-__host__ __device__ constexpr uint32_t tab_entries(uint32_t K) { return K > 1 ? 1u << (K - 1) : 1u; }
+// entries of the table of a 2^K-point sub-transform (at least one group)
+__host__ __device__ constexpr uint32_t tab_entries(uint32_t K) { return K > 3 ? 1u << (K - 1) : 8u; }
 
 // issue (without waiting) the copies of the table, which is laid out in global
 // memory as in shared memory
-__device__ __forceinline__ void issue_table_load(const PassArgs &a, uint4 *tab) {
+__device__ __forceinline__ void issue_table_load(const PassArgs &a, uint4 *tab, uint32_t nthreads) {
     const uint32_t units = 4 * tab_entries(a.K);
-    for (uint32_t u = threadIdx.x; u < units; u += blockDim.x) cp_async16(tab + u, a.w_stage + u);
+#pragma unroll 1
+    for (uint32_t u = threadIdx.x; u < units; u += nthreads) cp_async16(tab + u, a.w_stage + u);
 }
 
-// the factor at table slot s (h = entries)
-__device__ __forceinline__ void lds_factor(Factor &f, const uint4 *tab, uint32_t h, uint32_t s) {
-    lds_elem(f.w, tab, tab + h, s);
-    lds_elem(f.wq, tab + 2 * h, tab + 3 * h, s);
+// the factor at unit u of the table
+__device__ __forceinline__ void lds_factor(Factor &f, const uint4 *tab, uint32_t u) {
+    lds_elem(f.w, tab, u);
+    lds_elem(f.wq, tab, u + 16);
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // How a tile's stages run: two at a time, four elements a thread (radix 4), or
 // one by one, one butterfly a thread (radix 2); or either by the thread count.
 enum Steps { RADIX4 = 1, RADIX2 = 2, EITHER = 3 };
 
-// x <- x + y, t = x - y + r (for the product): the sum and lazy difference of
-// a butterfly
+// x <- x + y, t = x - y (for the product): a butterfly but for its product
 template <class F>
 __device__ __forceinline__ void sum_diff(uint32_t x[8], uint32_t t[8], const uint32_t y[8]) {
-    sub_lazy<F>(t, x, y);
-    add<F>(x, x, y);
+    diff_loose<F>(t, x, y);
+    add_loose<F>(x, x, y);
+}
+
+// x <- x + y, y <- x - y: a butterfly with twiddle 1
+template <class F>
+__device__ __forceinline__ void sum_sub(uint32_t x[8], uint32_t y[8]) {
+    uint32_t t[8];
+    sub_loose<F>(t, x, y);
+    add_loose<F>(x, x, y);
+#pragma unroll
+    for (int k = 0; k < 8; k++) y[k] = t[k];
 }
 
 // One stage, pairs at distance h, one butterfly after the other.
 template <class F>
-__device__ __forceinline__ void radix2_stage(uint4 *s_lo, uint4 *s_hi, const uint4 *tab, uint32_t h,
+__device__ __forceinline__ void radix2_stage(uint4 *buf, const uint4 *tab, uint32_t h,
                                              uint32_t K, uint32_t lc, uint32_t tid,
                                              uint32_t nthreads) {
-    const uint32_t N = 1u << K, CN = N << lc, step = row_slot(h);
+    const uint32_t N = 1u << K, CN = N << lc, step = row_unit(h);
     const uint32_t shift = K - 1 - (31 - __clz(h));  // entry j 2^stage
     for (uint32_t bk = tid; tid < nthreads && bk < (CN >> 1); bk += nthreads) {
         const uint32_t cc = bk >> (K - 1), b = bk & ((N >> 1) - 1), j = b & (h - 1);
-        const uint32_t s0 = smem_slot(cc, ((b ^ j) << 1) | j, K, lc), s1 = s0 ^ step;
+        const uint32_t s0 = smem_unit(cc, ((b ^ j) << 1) | j, K, lc), s1 = s0 ^ step;
         uint32_t x[8], y[8], t[8];
         Factor w;
-        lds_elem(x, s_lo, s_hi, s0);
-        lds_elem(y, s_lo, s_hi, s1);
-        lds_factor(w, tab, N >> 1, tab_slot(j << shift));
+        lds_elem(x, buf, s0);
+        lds_elem(y, buf, s1);
+        lds_factor(w, tab, tab_unit(j << shift));
         sum_diff<F>(x, t, y);
         mul_factor<F>(t, t, w);
-        sts_elem(s_lo, s_hi, s0, x);
-        sts_elem(s_lo, s_hi, s1, t);
+        sts_elem(buf, s0, x);
+        sts_elem(buf, s1, t);
     }
 }
 
@@ -327,8 +415,6 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
     const uint32_t N = 1u << K;
     const uint32_t C = 1u << lc;
     const uint32_t CN = C << K;
-    uint4 *s_lo = buf;
-    uint4 *s_hi = buf + CN;
     const uint32_t tid = threadIdx.x;
     const bool active = tid < nthreads;
 
@@ -339,9 +425,9 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
             uint32_t d, cc;
             if (a.last) { d = e & (N - 1); cc = e >> K; }
             else        { cc = e & (C - 1); d = e >> lc; }
-            const uint32_t s = smem_slot(cc, d, K, lc);
+            const uint32_t s = smem_unit(cc, d, K, lc);
             uint32_t x[8];
-            lds_elem(x, s_lo, s_hi, s);
+            lds_elem(x, buf, s);
             if (a.pw_b) {
                 const size_t g = tile_src(a, tile, d, cc);
                 uint32_t v[8], u[8];
@@ -355,53 +441,68 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
                 ldg_factor(f, a.pre + 4 * size_t(d));
                 mul_factor<F>(x, x, f);
             }
-            sts_elem(s_lo, s_hi, s, x);
+            sts_elem(buf, s, x);
         }
         __syncthreads();
+    }
+
+    // the thread's entries of the big table are wanted in the last step: into L2
+    const uint32_t cc_out = tid & (C - 1), d_out = (tid >> lc) << 2;
+    if (K >= 2 && !a.last && !a.otf && active && tid < (CN >> 2)) {
+        const OutRows o = out_rows<4>(a, tile, d_out, cc_out);
+#pragma unroll
+        for (int i = 0; i < 4; i++) prefetch_l2(o.f + i * o.fstep);
     }
 
     // ---- stages 0 .. K-3
     if (STEPS == RADIX2 || (STEPS == EITHER && nthreads > (CN >> 2))) {
         for (uint32_t h = N >> 1; h >= 4; h >>= 1) {
-            radix2_stage<F>(s_lo, s_hi, tab, h, K, lc, tid, nthreads);
+            radix2_stage<F>(buf, tab, h, K, lc, tid, nthreads);
             __syncthreads();
         }
     } else if (K > 2) {
         uint32_t q = N >> 2;  // distance of a radix-4 step's rows
         if (K & 1u) {
-            radix2_stage<F>(s_lo, s_hi, tab, N >> 1, K, lc, tid, nthreads);
+            radix2_stage<F>(buf, tab, N >> 1, K, lc, tid, nthreads);
             __syncthreads();
             q >>= 1;
         }
+        // the thread's group, and its column's part of the units
+        const uint32_t g0 = tid & ((N >> 2) - 1), c0 = col_unit(tid >> (K - 2), K, lc);
         uint32_t shift = K & 1u;  // the step's first stage: entries j 2^shift and (j + q) 2^shift
+#pragma unroll 1
         for (; q > 1; q >>= 2, shift += 2) {
             // rows i0 + {0, q, 2q, 3q}: the stage of distance 2q, then of distance q
-            const uint32_t x1 = row_slot(q), x2 = row_slot(2 * q), xt = tab_slot(q << shift);
-            for (uint32_t g = tid; active && g < (CN >> 2); g += nthreads) {
-                const uint32_t cc = g >> (K - 2), b = g & ((N >> 2) - 1), j = b & (q - 1);
-                const uint32_t s0 = smem_slot(cc, ((b ^ j) << 2) | j, K, lc);
-                const uint32_t ta = tab_slot(j << shift), tb = tab_slot(j << (shift + 1));
+            const uint32_t x1 = row_unit(q), x2 = row_unit(2 * q), xt = tab_unit(q << shift);
+            uint32_t g = tid, b = g0, c = c0;
+            while (active && g < (CN >> 2)) {
+                const uint32_t j = b & (q - 1);
+                const uint32_t u0 = c ^ row_unit(4 * b - 3 * j);
+                const uint32_t ta = tab_unit(j << shift), tb = tab_unit(j << (shift + 1));
                 uint32_t v0[8], v1[8], v2[8], v3[8], t[8];
                 Factor w;
-                lds_elem(v0, s_lo, s_hi, s0);
-                lds_elem(v2, s_lo, s_hi, s0 ^ x2);
-                lds_factor(w, tab, N >> 1, ta);
+                lds_elem(v0, buf, u0);
+                lds_elem(v2, buf, u0 ^ x2);
+                lds_factor(w, tab, ta);
                 sum_diff<F>(v0, t, v2);
                 mul_factor<F>(v2, t, w);
-                lds_elem(v1, s_lo, s_hi, s0 ^ x1);
-                lds_elem(v3, s_lo, s_hi, s0 ^ x1 ^ x2);
-                lds_factor(w, tab, N >> 1, ta ^ xt);
+                lds_elem(v1, buf, u0 ^ x1);
+                lds_elem(v3, buf, u0 ^ x1 ^ x2);
+                lds_factor(w, tab, ta ^ xt);
                 sum_diff<F>(v1, t, v3);
                 mul_factor<F>(v3, t, w);
-                lds_factor(w, tab, N >> 1, tb);
+                lds_factor(w, tab, tb);
                 sum_diff<F>(v0, t, v1);
-                sts_elem(s_lo, s_hi, s0, v0);
+                sts_elem(buf, u0, v0);
                 mul_factor<F>(v1, t, w);
-                sts_elem(s_lo, s_hi, s0 ^ x1, v1);
+                sts_elem(buf, u0 ^ x1, v1);
                 sum_diff<F>(v2, t, v3);
-                sts_elem(s_lo, s_hi, s0 ^ x2, v2);
+                sts_elem(buf, u0 ^ x2, v2);
                 mul_factor<F>(v3, t, w);
-                sts_elem(s_lo, s_hi, s0 ^ x1 ^ x2, v3);
+                sts_elem(buf, u0 ^ x1 ^ x2, v3);
+                g += nthreads;
+                b = g & ((N >> 2) - 1);
+                c = col_unit(g >> (K - 2), K, lc);
             }
             // at q <= 32 a warp's groups, 32 consecutive ones, are made of rows
             // of its own, at this step and the next: only the last step (columns
@@ -413,116 +514,140 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
 
     // ---- last two stages as radix-4 on rows d0..d0+3, factors and store
     // (columns fastest: C-element runs in global memory)
-    const bool scaled = a.last ? a.post != nullptr : true;
     if (K >= 2) {
         Factor w4;
-        lds_factor(w4, tab, N >> 1, tab_slot(N >> 2));  // w_N^(N/4) = w_4
+        lds_factor(w4, tab, tab_unit(N >> 2));  // w_N^(N/4) = w_4
         for (uint32_t qd = tid; active && qd < (CN >> 2); qd += nthreads) {
             const uint32_t cc = qd & (C - 1);
             const uint32_t d0 = (qd >> lc) << 2;
             uint32_t x0[8], x1[8], x2[8], x3[8], t[8];
             // rows d0 + i (d0 a multiple of 4) share the swizzle term: their
-            // slots are the first one's with i in the low two bits
-            const uint32_t s0 = smem_slot(cc, d0, K, lc), s1 = s0 ^ 1u, s2 = s0 ^ 2u, s3 = s0 ^ 3u;
-            lds_elem(x0, s_lo, s_hi, s0);
-            lds_elem(x1, s_lo, s_hi, s1);
-            lds_elem(x2, s_lo, s_hi, s2);
-            lds_elem(x3, s_lo, s_hi, s3);
+            // units are the first one's with i in the low two bits
+            const uint32_t u0 = smem_unit(cc, d0, K, lc);
+            lds_elem(x1, buf, u0 ^ 1u);
+            lds_elem(x3, buf, u0 ^ 3u);
+            lds_elem(x0, buf, u0);
+            lds_elem(x2, buf, u0 ^ 2u);
             // stage K-2: pairs (0,2) with twiddle 1, (1,3) with w_4
-            sub<F>(t, x0, x2);
-            add<F>(x0, x0, x2);
-#pragma unroll
-            for (int k = 0; k < 8; k++) x2[k] = t[k];
             sum_diff<F>(x1, t, x3);
             mul_factor<F>(x3, t, w4);
+            sum_sub<F>(x0, x2);
             // stage K-1: pairs (0,1), (2,3), twiddle 1
-            sub<F>(t, x0, x1);
-            add<F>(x0, x0, x1);
-            if (!scaled) {
-                st_elem(a.out + 2 * tile_dst(a, tile, d0, cc), x0);
-                st_elem(a.out + 2 * tile_dst(a, tile, d0 + 1, cc), t);
-                sub<F>(t, x2, x3);
-                add<F>(x2, x2, x3);
-                st_elem(a.out + 2 * tile_dst(a, tile, d0 + 2, cc), x2);
-                st_elem(a.out + 2 * tile_dst(a, tile, d0 + 3, cc), t);
-                continue;
-            }
-            // through the thread's own slots into a loop with one product
-            sts_elem(s_lo, s_hi, s0, x0);
-            sts_elem(s_lo, s_hi, s1, t);
-            sub<F>(t, x2, x3);
-            add<F>(x2, x2, x3);
-            sts_elem(s_lo, s_hi, s2, x2);
-            sts_elem(s_lo, s_hi, s3, t);
-#pragma unroll 1
-            for (uint32_t i = 0; i < 4; i++) {
-                uint32_t x[8];
-                lds_elem(x, s_lo, s_hi, s0 ^ i);
-                scale_and_store<F>(x, a, tile, d0 + i, cc);
+            sum_sub<F>(x0, x1);
+            sum_sub<F>(x2, x3);
+            const OutRows o = out_rows<4>(a, tile, d0, cc);
+            if (a.last && !o.f) {
+                // no factor: below r, and out (rows in bit-reversed order)
+                reduce_once<F>(x0);
+                st_elem8(o.out, x0);
+                reduce_once<F>(x1);
+                st_elem8(o.out + 4 * o.step, x1);
+                reduce_once<F>(x2);
+                st_elem8(o.out + 2 * o.step, x2);
+                reduce_once<F>(x3);
+                st_elem8(o.out + 6 * o.step, x3);
+            } else {
+                // through the thread's own slots into a loop over the rows
+                sts_elem(buf, u0, x0);
+                sts_elem(buf, u0 ^ 1u, x1);
+                sts_elem(buf, u0 ^ 2u, x2);
+                sts_elem(buf, u0 ^ 3u, x3);
+                scale_and_store<F, 4>(a, buf, u0, o, tile, d0, cc);
             }
         }
     } else {
         // N = 2: one radix-2 butterfly per column
         for (uint32_t cc = tid; active && cc < C; cc += nthreads) {
-            uint32_t x0[8], x1[8], t[8];
-            const uint32_t s0 = smem_slot(cc, 0, K, lc), s1 = smem_slot(cc, 1, K, lc);
-            lds_elem(x0, s_lo, s_hi, s0);
-            lds_elem(x1, s_lo, s_hi, s1);
-            sub<F>(t, x0, x1);
-            add<F>(x0, x0, x1);
-            sts_elem(s_lo, s_hi, s0, x0);
-            sts_elem(s_lo, s_hi, s1, t);
-#pragma unroll 1
-            for (uint32_t i = 0; i < 2; i++) {
-                uint32_t x[8];
-                lds_elem(x, s_lo, s_hi, s0 + i);
-                scale_and_store<F>(x, a, tile, i, cc);
+            uint32_t x0[8], x1[8];
+            const uint32_t u0 = smem_unit(cc, 0, K, lc);
+            lds_elem(x0, buf, u0);
+            lds_elem(x1, buf, u0 ^ 1u);
+            sum_sub<F>(x0, x1);
+            const OutRows o = out_rows<2>(a, tile, 0, cc);
+            if (a.last && !o.f) {
+                reduce_once<F>(x0);
+                st_elem8(o.out, x0);
+                reduce_once<F>(x1);
+                st_elem8(o.out + 2 * o.step, x1);
+            } else {
+                sts_elem(buf, u0, x0);
+                sts_elem(buf, u0 ^ 1u, x1);
+                scale_and_store<F, 2>(a, buf, u0, o, tile, 0, cc);
             }
         }
     }
 }
 
-// threads per block for a tile of C x 2^K elements: one per radix-4 group,
-// at most 256
-__host__ __device__ constexpr uint32_t pass_threads(uint32_t K, uint32_t lc) {
-    return ((K >= 2 ? (1u << (K + lc - 2)) : (1u << lc)) < 256u)
-               ? (K >= 2 ? (1u << (K + lc - 2)) : (1u << lc))
-               : 256u;
-}
-
-// threads per block for schedule variant v: variant 5 doubles the count (one
-// butterfly per thread per stage), still at most 256
+// threads per block of schedule variant v for a tile of C x 2^K elements: one
+// per four elements (variant 5: two, one butterfly a thread and stage), at most
+// what the variant's kernel is compiled for
+__host__ __device__ constexpr uint32_t pass_max_threads(int v) { return v == 1 || v == 7 ? 128u : 256u; }
 __host__ __device__ constexpr uint32_t pass_threads_for(uint32_t K, uint32_t lc, int v) {
-    return v == 5 && K >= 2 && pass_threads(K, lc) < 256u ? 2u * pass_threads(K, lc)
-                                                           : pass_threads(K, lc);
+    const uint32_t t = K >= 2 ? 1u << (K + lc - (v == 5 ? 1 : 2)) : 1u << lc;
+    return t < pass_max_threads(v) ? t : pass_max_threads(v);
 }
 
-// One pass.  MIN_BLOCKS: blocks of 256 threads an SM the register budget is
-// for (2: 128 registers, 3: 80, 4: 64).
-template <class F, int MIN_BLOCKS, Steps STEPS>
-__global__ void __launch_bounds__(256, MIN_BLOCKS) ntt_pass_kernel(const PassArgs a) {
+// What a pass kernel is compiled for.  ANY: every argument is a runtime value.
+// The others: a digit of K bits in tiles of fixed_cols(K) columns; a strided pass
+// with precomputed twiddles, its input without factors (STRIDED) or with
+// (STRIDED_PRE), or with twiddles on the fly (STRIDED_OTF); the last pass without
+// output factors (LAST) or with (LAST_POST).  With these fixed the index
+// arithmetic of a tile shrinks: 803 -> 692 instructions an element in the last
+// pass of 2^22, which was 691 us and is 642 (BLS12-381, digits 8, 7, 7).  (With
+// the digit alone fixed and the factors left to the arguments 2^22 took 648, 2^12
+// to 2^16 a tenth longer.)
+enum Kind { ANY, STRIDED, STRIDED_PRE, STRIDED_OTF, LAST, LAST_POST, NUM_KINDS };
+
+// log2 of the columns of the tiles of the compiled digits: two, so that global
+// memory is read and written in 64-byte pieces; one where two make a tile and
+// table of which only one would fit an SM
+__host__ __device__ constexpr int fixed_cols(int K) { return K < 10 ? 1 : 0; }
+
+template <int K, Kind KIND>
+__device__ __forceinline__ void fix_args(PassArgs &a) {
+    if (KIND == ANY) return;
+    a.K = K;
+    a.log_cols = fixed_cols(K);
+    a.last = KIND == LAST || KIND == LAST_POST;
+    a.otf = KIND == STRIDED_OTF;
+    a.pw_b = a.pw_c = nullptr;
+    if (KIND != STRIDED_PRE) a.pre = nullptr;
+    if (KIND != LAST_POST) a.post = nullptr;
+}
+
+// One pass.  The register budget is for BLOCKS blocks of THREADS threads an SM.
+template <class F, int THREADS, int BLOCKS, Steps STEPS, int K, Kind KIND>
+__global__ void __launch_bounds__(THREADS, BLOCKS) ntt_pass_kernel(const PassArgs args) {
     extern __shared__ uint4 smem[];
-    // Two tile buffers when the block has more than one tile: the copies of its
-    // next tile are in flight while the current one is computed.
-    const uint32_t CN = 1u << (a.K + a.log_cols);
+    PassArgs a = args;
+    fix_args<K, KIND>(a);
+    const uint32_t nthreads = KIND == ANY ? blockDim.x : THREADS;
+    const uint32_t units = tile_units(1u << (a.K + a.log_cols));
     uint4 *tab = smem, *buf = smem + 4 * tab_entries(a.K);
-    uint32_t tile = blockIdx.x;
-    issue_table_load(a, tab);  // (a plan's table: no pass writes it)
+    issue_table_load(a, tab, nthreads);  // (a plan's table: no pass writes it)
     // Passes after the first are launched as programmatic dependents of the
     // pass before, and wait here until that pass has completed and its writes
     // are visible (launched without that attribute, the wait returns at once).
     // A block lets the next pass launch when it starts its last tile, so the
     // next pass's blocks take SM places only as this grid winds down.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tile < a.num_tiles) issue_tile_load(a, buf, tile, blockDim.x);
-    for (uint32_t cur = 0; tile < a.num_tiles; tile += gridDim.x, cur ^= 2 * CN) {
-        cp_async_wait_all();
-        // the tile is there, and every thread is done with the other buffer
-        __syncthreads();
-        const uint32_t next = tile + gridDim.x;
-        if (next < a.num_tiles) issue_tile_load(a, buf + (cur ^ (2 * CN)), next, blockDim.x);
+    uint32_t tile = a.num_tiles;  // the tile to compute (none yet)
+    // Two tile buffers when the block has more than one tile: the copies of its
+    // next tile are in flight while the current one is computed.
+    uint4 *cur = buf + units, *other = buf;
+#pragma unroll 1
+    for (uint32_t fetch = blockIdx.x;; fetch += gridDim.x) {
+        if (fetch < a.num_tiles) issue_tile_load(a, other, fetch, nthreads);
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        run_tile<F, STEPS>(a, tab, buf + cur, tile, blockDim.x);
+        if (tile < a.num_tiles) run_tile<F, STEPS>(a, tab, cur, tile, nthreads);
+        if (fetch >= a.num_tiles) break;
+        cp_async_wait_all();
+        // the fetched tile is there, and every thread is done with the other one
+        __syncthreads();
+        tile = fetch;
+        uint4 *const t = cur;
+        cur = other;
+        other = t;
     }
 }
 

@@ -197,14 +197,15 @@ static zkntt_status fill_uniform(zkntt_field field, void *d, size_t n) {
     return ZKNTT_OK;
 }
 
-// Candidate schedules for one digit split: both twiddle modes, variants
-// 1 .. TUNED_VARIANTS (6 and 7 were measured slower than 3 and 1 at every size
-// and stay explicit options), column caps 3..1.
+// Candidate schedules for one digit split: both twiddle modes, the variants of
+// different kernels (1, 2 and 5; the other numbers share theirs or a smaller
+// register budget that was slower at every size), column caps 1, 0, 2 and 3 (the
+// kernels compiled for a digit first).
 static void split_candidates(int log_n, const std::vector<int> &d, std::vector<zkntt_plan_options> &out) {
     const int p = int(d.size());
     for (int mode : {ZKNTT_TWIDDLE_PRECOMP, ZKNTT_TWIDDLE_OTF})
-        for (int ilp = 1; ilp <= TUNED_VARIANTS; ilp++)
-            for (int cap = 3; cap >= 1; cap--) {
+        for (int cap : {1, 0, 2, 3})
+            for (int ilp : {1, 2, 5}) {
                 if (p == 1 && (mode == ZKNTT_TWIDDLE_OTF || cap != 3)) continue;
                 zkntt_plan_options o;
                 memset(&o, 0, sizeof o);
@@ -216,6 +217,7 @@ static void split_candidates(int log_n, const std::vector<int> &d, std::vector<z
                     o.digit_bits[i] = d[i];
                     int span = (i == p - 1) ? hi : (log_n - hi - d[i]);
                     int lc = std::min({cap, MAX_DIGIT_BITS - d[i], span});
+                    if (d[i] == 10 && cap == 1) lc = 0;
                     o.cols_per_cta[i] = 1 << std::max(0, lc);
                     hi += d[i];
                 }
@@ -281,23 +283,12 @@ extern "C" zkntt_status zkntt_tune(zkntt_field field, int log_n, zkntt_dir dir, 
     };
 
     // Stage 1: every digit split with one representative schedule (precomputed
-    // tables; for small sizes the variant with twice the threads and wider
-    // tiles, else the 64-register variant with 2-column tiles).
+    // tables, two-column tiles, one column for digits of 10 bits).
     std::vector<std::pair<double, size_t>> ranked;
     for (size_t si = 0; si < all_splits.size() && result == ZKNTT_OK; si++) {
         std::vector<zkntt_plan_options> c;
         split_candidates(log_n, all_splits[si], c);
-        const int want_ilp = log_n <= 16 ? 5 : 3, want_cap = log_n <= 16 ? 2 : 1;
-        zkntt_plan_options rep = c.front();
-        for (const auto &o : c) {
-            int cap = 0;
-            for (int i = 0; i < o.num_passes; i++) cap = std::max(cap, o.cols_per_cta[i]);
-            if (o.twiddle_mode == ZKNTT_TWIDDLE_PRECOMP && o.ilp == want_ilp &&
-                cap <= (1 << want_cap)) {
-                rep = o;
-                break;
-            }
-        }
+        const zkntt_plan_options rep = c.front();
         const double ms = all_splits.size() > 1 ? time_one(rep, 3) : 0.0;
         if (ms >= 0) ranked.push_back({ms, si});
     }

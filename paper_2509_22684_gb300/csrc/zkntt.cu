@@ -301,6 +301,12 @@ zkntt_status device_info(DeviceInfo **out) {
                 ZK_CHECK(cudaFuncSetAttribute(field_kernels(f).pass[ilp],
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               PASS_MAX_SMEM));
+        for (int f = 0; f < NUM_FIELDS; f++)
+            for (const auto &by_kind : field_kernels(f).fixed)
+                for (const void *k : by_kind)
+                    if (k)
+                        ZK_CHECK(cudaFuncSetAttribute(
+                            k, cudaFuncAttributeMaxDynamicSharedMemorySize, PASS_MAX_SMEM));
         for (int f = 0; f < NUM_FIELDS; f++) {
             ZK_CHECK(cudaFuncSetAttribute(batch_kernel_ptr(f),
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -369,6 +375,7 @@ zkntt_status pool_alloc(void **p, size_t bytes, cudaStream_t s) {
 struct PassPlan {
     int K = 0, lo_bits = 0, hi_bits = 0, log_cols = 0, ilp = 1;
     int threads = 0, grid = 0;
+    const void *kernel = nullptr;
     uint32_t num_tiles = 0;
     size_t smem = 0;
     uint4 *w_stage = nullptr, *tw = nullptr, *w_hi = nullptr, *w_lo = nullptr, *fl = nullptr,
@@ -610,14 +617,31 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         ps.num_tiles = last ? (uint32_t(1) << (ps.hi_bits - lc))
                             : (uint32_t(1) << (ps.hi_bits + ps.lo_bits - lc));
         ps.threads = int(pass_threads_for(uint32_t(ps.K), uint32_t(lc), ilp));
-        // the twiddle table, and two tile buffers unless every block has one tile
-        const size_t tile_bytes = size_t(32) << (ps.K + lc);
+        ps.kernel = field_kernels(P->field).pass[ilp];
+        // a kernel compiled for this digit, where there is one and its tile is the
+        // schedule's
+        const bool scaled_in = i == 0 && coset && !inverse;
+        const bool scaled_out = (coset && inverse) || (p == 1 && !(out_scale == F.one));
+        Kind kind = ANY;
+        if (last) {
+            if (!scaled_in) kind = scaled_out ? LAST_POST : LAST;
+        } else if (mode == ZKNTT_TWIDDLE_OTF) {
+            if (!scaled_in) kind = STRIDED_OTF;
+        } else {
+            kind = scaled_in ? STRIDED_PRE : STRIDED;
+        }
+        const void *fixed = field_kernels(P->field).fixed[ps.K][kind];
+        if (ilp != 5 && lc == fixed_cols(ps.K) && fixed) {
+            ps.kernel = fixed;
+            ps.threads = 1 << (ps.K + lc - 2);
+        }
+        // the twiddle table and the tile buffers: one will do if every block has one tile
+        const size_t tile_bytes = size_t(16) * tile_units(1u << (ps.K + lc));
         const size_t table_bytes = size_t(64) * tab_entries(uint32_t(ps.K));
         int nb = 0;
-        for (int buffers = 1; buffers <= 2; buffers++) {
-            ps.smem = table_bytes + buffers * tile_bytes;
-            ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &nb, field_kernels(P->field).pass[ps.ilp], ps.threads, ps.smem));
+        for (int n = 1; n <= 2; n++) {
+            ps.smem = table_bytes + n * tile_bytes;
+            ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, ps.kernel, ps.threads, ps.smem));
             nb = std::max(nb, 1);
             if (ps.num_tiles <= uint64_t(nb) * dev->sms) break;
         }
@@ -627,22 +651,22 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         const E8 wn_i = hpow(F, w, uint64_t(1) << ps.hi_bits);          // root of order n_i
         const E8 wN = hpow(F, wn_i, uint64_t(1) << ps.lo_bits);         // root of order N_i
         {
-            // (in four planes of 16-byte quarters, as the kernels keep it in
-            // shared memory)
+            // (in groups of eight, quarter by quarter, as the kernels keep them
+            // in shared memory)
             const uint32_t h = tab_entries(uint32_t(ps.K));
             const std::vector<E8> all = powers(F, wN, h, F.one);
-            std::vector<uint32_t> planes(size_t(h) * 16);
+            std::vector<uint32_t> units(size_t(h) * 16);
             for (uint32_t e = 0; e < h; e++) {
                 const HFactor f = hfactor(F, all[e]);
-                uint32_t q[16];
-                memcpy(q, f.w.data(), 32);
-                memcpy(q + 8, f.wq.data(), 32);
-                for (int p4 = 0; p4 < 4; p4++)
-                    memcpy(&planes[(size_t(p4) * h + tab_slot(e)) * 4], q + 4 * p4, 16);
+                uint32_t *u = &units[size_t(tab_unit(e)) * 4];
+                memcpy(u, f.w.data(), 16);
+                memcpy(u + 32, f.w.data() + 4, 16);
+                memcpy(u + 64, f.wq.data(), 16);
+                memcpy(u + 96, f.wq.data() + 4, 16);
             }
             st = dalloc(P, &ps.w_stage, 2 * size_t(h));
             if (st != ZKNTT_OK) return st;
-            st = from_cuda(cudaMemcpy(ps.w_stage, planes.data(), size_t(h) * 64, cudaMemcpyHostToDevice));
+            st = from_cuda(cudaMemcpy(ps.w_stage, units.data(), size_t(h) * 64, cudaMemcpyHostToDevice));
             if (st != ZKNTT_OK) return st;
         }
 
@@ -763,7 +787,6 @@ zkntt_status check_plan_device(const zkntt_plan_s *P) {
 
 zkntt_status run_passes(const zkntt_plan_s *P, const void *in, void *out, void *scratch,
                         cudaStream_t s) {
-    const FieldKernels &kk = field_kernels(P->field);
     for (int i = 0; i < P->passes; i++) {
         const void *src = (i == 0) ? in : scratch;
         void *dst = (i == P->passes - 1) ? out : scratch;
@@ -774,7 +797,7 @@ zkntt_status run_passes(const zkntt_plan_s *P, const void *in, void *out, void *
             // the first pass is ordered after all earlier work on the stream
             // (which may write `in`); plans of the two-butterfly variant keep
             // plain launches throughout (measured 1-7% slower as dependents)
-            ZK_CHECK(cudaLaunchKernel(kk.pass[ps.ilp], dim3(ps.grid), dim3(ps.threads), args, ps.smem, s));
+            ZK_CHECK(cudaLaunchKernel(ps.kernel, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s));
             continue;
         }
         // later passes depend only on the pass before: a programmatic
@@ -790,7 +813,7 @@ zkntt_status run_passes(const zkntt_plan_s *P, const void *in, void *out, void *
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        ZK_CHECK(cudaLaunchKernelExC(&cfg, kk.pass[ps.ilp], args));
+        ZK_CHECK(cudaLaunchKernelExC(&cfg, ps.kernel, args));
     }
     return ZKNTT_OK;
 }
@@ -984,7 +1007,7 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
         size_t tile_bytes = 0, table_bytes = 0;
         for (int k = 0; k < int(segs.size()); k++) {
             const PassArgs &a = tab->seg[k].a;
-            tile_bytes = std::max(tile_bytes, size_t(32) << (a.K + a.log_cols));
+            tile_bytes = std::max(tile_bytes, size_t(16) * tile_units(1u << (a.K + a.log_cols)));
             table_bytes = std::max(table_bytes, size_t(64) * tab_entries(a.K));
         }
         tab->table_units = uint32_t(table_bytes / 16);
