@@ -590,7 +590,7 @@ __host__ __device__ constexpr uint32_t pass_threads_for(uint32_t K, uint32_t lc,
 // What a pass kernel is compiled for.  ANY: every argument is a runtime value.
 // The others: a digit of K bits in tiles of fixed_cols(K) columns; a strided pass
 // with precomputed twiddles, its input without factors (STRIDED) or with
-// (STRIDED_PRE), or with twiddles on the fly (STRIDED_OTF); the last pass without
+// (STRIDED_PRE: input scales or the pointwise step), or with twiddles on the fly (STRIDED_OTF); the last pass without
 // output factors (LAST) or with (LAST_POST).  With these fixed the index
 // arithmetic of a tile shrinks: 803 -> 692 instructions an element in the last
 // pass of 2^22, which was 691 us and is 642 (BLS12-381, digits 8, 7, 7).  (With
@@ -610,8 +610,7 @@ __device__ __forceinline__ void fix_args(PassArgs &a) {
     a.log_cols = fixed_cols(K);
     a.last = KIND == LAST || KIND == LAST_POST;
     a.otf = KIND == STRIDED_OTF;
-    a.pw_b = a.pw_c = nullptr;
-    if (KIND != STRIDED_PRE) a.pre = nullptr;
+    if (KIND != STRIDED_PRE) a.pre = a.pw_b = a.pw_c = nullptr;
     if (KIND != LAST_POST) a.post = nullptr;
 }
 

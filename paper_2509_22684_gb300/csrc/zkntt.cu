@@ -372,12 +372,18 @@ zkntt_status pool_alloc(void **p, size_t bytes, cudaStream_t s) {
 }  // namespace
 
 // ---------------------------------------------------------------------------
+// how a pass is launched
+struct PassLaunch {
+    const void *kernel = nullptr;
+    int threads = 0, grid = 0;
+    size_t smem = 0;
+};
+
 struct PassPlan {
     int K = 0, lo_bits = 0, hi_bits = 0, log_cols = 0, ilp = 1;
-    int threads = 0, grid = 0;
-    const void *kernel = nullptr;
     uint32_t num_tiles = 0;
-    size_t smem = 0;
+    PassLaunch run;      // the pass
+    PassLaunch run_pw;   // first pass: with the pointwise step on its input
     uint4 *w_stage = nullptr, *tw = nullptr, *w_hi = nullptr, *w_lo = nullptr, *fl = nullptr,
           *fd = nullptr;
     int tw_bits = 0, split_bits = 0;
@@ -513,6 +519,33 @@ zkntt_status split_tables(zkntt_plan_s *P, const HostField &F, const E8 &base, i
     return put(P, F, hi, powers(F, step, size_t(1) << (bits - sp), F.one));
 }
 
+// Kernel, block and grid of a pass whose sizes are set: a kernel compiled for
+// this digit and kind, where there is one and its tile is the schedule's, else
+// the variant's kernel of runtime sizes.
+zkntt_status set_launch(const PassPlan *ps, PassLaunch *r, int field, Kind kind, int sms) {
+    const FieldKernels &kk = field_kernels(field);
+    const void *fixed = kk.fixed[ps->K][kind];
+    if (ps->ilp != 5 && ps->log_cols == fixed_cols(ps->K) && fixed) {
+        r->kernel = fixed;
+        r->threads = 1 << (ps->K + ps->log_cols - 2);
+    } else {
+        r->kernel = kk.pass[ps->ilp];
+        r->threads = int(pass_threads_for(uint32_t(ps->K), uint32_t(ps->log_cols), ps->ilp));
+    }
+    // the twiddle table and the tile buffers: one will do if every block has one tile
+    const size_t tile_bytes = size_t(16) * tile_units(1u << (ps->K + ps->log_cols));
+    const size_t table_bytes = size_t(64) * tab_entries(uint32_t(ps->K));
+    int nb = 0;
+    for (int n = 1; n <= 2; n++) {
+        r->smem = table_bytes + n * tile_bytes;
+        ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, r->kernel, r->threads, r->smem));
+        nb = std::max(nb, 1);
+        if (ps->num_tiles <= uint64_t(nb) * sms) break;
+    }
+    r->grid = int(std::min<uint64_t>(ps->num_tiles, uint64_t(nb) * sms));
+    return ZKNTT_OK;
+}
+
 zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
     const HostField &F = host_field(P->field);
     if (!F.ok) return ZKNTT_ECUDA;
@@ -616,36 +649,20 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         ps.ilp = ilp;
         ps.num_tiles = last ? (uint32_t(1) << (ps.hi_bits - lc))
                             : (uint32_t(1) << (ps.hi_bits + ps.lo_bits - lc));
-        ps.threads = int(pass_threads_for(uint32_t(ps.K), uint32_t(lc), ilp));
-        ps.kernel = field_kernels(P->field).pass[ilp];
-        // a kernel compiled for this digit, where there is one and its tile is the
-        // schedule's
         const bool scaled_in = i == 0 && coset && !inverse;
         const bool scaled_out = (coset && inverse) || (p == 1 && !(out_scale == F.one));
-        Kind kind = ANY;
+        Kind kind = ANY, kind_pw = ANY;
         if (last) {
             if (!scaled_in) kind = scaled_out ? LAST_POST : LAST;
         } else if (mode == ZKNTT_TWIDDLE_OTF) {
             if (!scaled_in) kind = STRIDED_OTF;
         } else {
             kind = scaled_in ? STRIDED_PRE : STRIDED;
+            kind_pw = STRIDED_PRE;
         }
-        const void *fixed = field_kernels(P->field).fixed[ps.K][kind];
-        if (ilp != 5 && lc == fixed_cols(ps.K) && fixed) {
-            ps.kernel = fixed;
-            ps.threads = 1 << (ps.K + lc - 2);
-        }
-        // the twiddle table and the tile buffers: one will do if every block has one tile
-        const size_t tile_bytes = size_t(16) * tile_units(1u << (ps.K + lc));
-        const size_t table_bytes = size_t(64) * tab_entries(uint32_t(ps.K));
-        int nb = 0;
-        for (int n = 1; n <= 2; n++) {
-            ps.smem = table_bytes + n * tile_bytes;
-            ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, ps.kernel, ps.threads, ps.smem));
-            nb = std::max(nb, 1);
-            if (ps.num_tiles <= uint64_t(nb) * dev->sms) break;
-        }
-        ps.grid = int(std::min<uint64_t>(ps.num_tiles, uint64_t(nb) * dev->sms));
+        st = set_launch(&ps, &ps.run, P->field, kind, dev->sms);
+        if (st == ZKNTT_OK && i == 0) st = set_launch(&ps, &ps.run_pw, P->field, kind_pw, dev->sms);
+        if (st != ZKNTT_OK) return st;
 
         // sub-transform twiddles w_N^e, e < N/2 (stage s uses w_N^(j 2^s))
         const E8 wn_i = hpow(F, w, uint64_t(1) << ps.hi_bits);          // root of order n_i
@@ -785,35 +802,39 @@ zkntt_status check_plan_device(const zkntt_plan_s *P) {
     return cur == P->device ? ZKNTT_OK : ZKNTT_EINVAL;
 }
 
+// pw_b, pw_c (both or neither): the transform of in * pw_b - pw_c
 zkntt_status run_passes(const zkntt_plan_s *P, const void *in, void *out, void *scratch,
-                        cudaStream_t s) {
+                        cudaStream_t s, const void *pw_b = nullptr, const void *pw_c = nullptr) {
     for (int i = 0; i < P->passes; i++) {
         const void *src = (i == 0) ? in : scratch;
         void *dst = (i == P->passes - 1) ? out : scratch;
         PassArgs a = pass_args(P, i, src, dst);
+        if (i == 0) {
+            a.pw_b = static_cast<const uint4 *>(pw_b);
+            a.pw_c = static_cast<const uint4 *>(pw_c);
+        }
         void *args[] = {&a};
-        const PassPlan &ps = P->ps[i];
-        if (i == 0 || ps.ilp == 2) {
+        const PassLaunch &r = (i == 0 && pw_b) ? P->ps[i].run_pw : P->ps[i].run;
+        if (i == 0) {
             // the first pass is ordered after all earlier work on the stream
-            // (which may write `in`); plans of the two-butterfly variant keep
-            // plain launches throughout (measured 1-7% slower as dependents)
-            ZK_CHECK(cudaLaunchKernel(ps.kernel, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s));
+            // (which may write `in`)
+            ZK_CHECK(cudaLaunchKernel(r.kernel, dim3(r.grid), dim3(r.threads), args, r.smem, s));
             continue;
         }
         // later passes depend only on the pass before: a programmatic
         // dependent launch overlaps their launch with its tail (the kernel
         // waits for the previous pass's completion before any memory access)
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(ps.grid);
-        cfg.blockDim = dim3(ps.threads);
-        cfg.dynamicSmemBytes = ps.smem;
+        cfg.gridDim = dim3(r.grid);
+        cfg.blockDim = dim3(r.threads);
+        cfg.dynamicSmemBytes = r.smem;
         cfg.stream = s;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        ZK_CHECK(cudaLaunchKernelExC(&cfg, ps.kernel, args));
+        ZK_CHECK(cudaLaunchKernelExC(&cfg, r.kernel, args));
     }
     return ZKNTT_OK;
 }
@@ -1078,6 +1099,13 @@ unsigned long long batch_timeout_ns() {
     if (ms == 0) ms = 2000;
     return ms * 1000000ull;
 }
+
+// From this size on the fused Groth16 sequence runs its transforms one after the
+// other as passes of the compiled kernels (each fills the GPU), below it as one
+// persistent launch, whose three independent transforms share the GPU.  Graph
+// replays, BLS12-381, persistent / passes: 2^16 109 / 117 us, 2^17 201 / 175,
+// 2^18 338 / 318, 2^20 1129 / 1189, 2^21 2536 / 2353, 2^22 5204 / 4745.
+constexpr int G16_PASSES_LOG_N = 17;
 
 // Groth16 plans per (field, log_n).  Separate form (the sequence as stated):
 // iNTT, coset NTT, coset iNTT.  Fused form: cosetNTT_g(iNTT(a)) is computed as
@@ -1413,6 +1441,19 @@ zkntt_status zkntt_groth16_h_ex(zkntt_field field, int log_n, const void *d_a, c
         if (st != ZKNTT_OK) return st;
         if (st2 != ZKNTT_OK) return st2;
         return zkntt_execute(G->cintt, d_h, d_h, s);
+    }
+    if (log_n >= G16_PASSES_LOG_N) {
+        const size_t need = scratch_bytes_of(G->ntt);
+        void *ps = nullptr;
+        if (need && (st = pool_alloc(&ps, need, s))) return st;
+        for (int k = 0; k < 3 && st == ZKNTT_OK; k++) st = run_passes(G->intt_gj, in[k], sv[k], ps, s);
+        for (int k = 0; k < 3 && st == ZKNTT_OK; k++) st = run_passes(G->ntt, sv[k], sv[k], ps, s);
+        if (st == ZKNTT_OK) st = run_passes(G->cintt_z, S0, d_h, ps, s, S1, S2);
+        if (ps) {
+            zkntt_status st2 = from_cuda(cudaFreeAsync(ps, s));
+            if (st == ZKNTT_OK) st = st2;
+        }
+        return st;
     }
     // fused: one persistent launch over the dependency graph
     //   jobs 0-2: cosetINTT_{g^-1}(a|b|c) -> S0|S1|S2   levels 0 .. p-1
