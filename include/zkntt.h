@@ -81,7 +81,7 @@ typedef struct {
     int ilp;               /* kernel variant: two stages at a time, four elements a thread, with
                               registers for 5 blocks of 128 threads per SM (1 and 7) or for
                               2 (2 and 4) or 3 (3 and 6) blocks of 256; 5 = one butterfly
-                              per thread per stage, registers for 4 blocks of 256 (for
+                              per thread per stage, registers for 2 blocks of 256 (for
                               small transforms); 0 = auto; outside 0..7 -> ZKNTT_EINVAL */
 } zkntt_plan_options;
 

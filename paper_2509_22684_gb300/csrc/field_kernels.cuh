@@ -16,6 +16,21 @@ const void *fixed_kernel() {
     return (const void *)&ntt_pass_kernel<F, T, B, RADIX4, K, KIND>;
 }
 
+// the same one butterfly a thread and stage, for small transforms: 128 registers
+template <class F, int K, Kind KIND>
+const void *wide_kernel() {
+    constexpr int T = 1 << (K + fixed_cols(K) - 1);
+    return (const void *)&ntt_pass_kernel<F, T, 512 / T, RADIX2, K, KIND>;
+}
+
+template <class F, int K>
+void set_wide(FieldKernels &k) {
+    k.wide[K][STRIDED] = wide_kernel<F, K, STRIDED>();
+    k.wide[K][STRIDED_PRE] = wide_kernel<F, K, STRIDED_PRE>();
+    k.wide[K][LAST] = wide_kernel<F, K, LAST>();
+    k.wide[K][LAST_POST] = wide_kernel<F, K, LAST_POST>();
+}
+
 template <class F, int K>
 void set_fixed(FieldKernels &k) {
     k.fixed[K][STRIDED] = fixed_kernel<F, K, STRIDED>();
@@ -28,11 +43,15 @@ void set_fixed(FieldKernels &k) {
 template <class F>
 FieldKernels make_field_kernels() {
     FieldKernels k = {};
-    // registers: 96 (variants 1 and 7), 128 (2 and 4), 80 (3 and 6), 64 (5)
+    // registers: 96 (variants 1 and 7), 128 (2, 4 and 5), 80 (3 and 6)
     k.pass[1] = k.pass[7] = (const void *)&ntt_pass_kernel<F, 128, 5, RADIX4, 0, ANY>;
     k.pass[2] = k.pass[4] = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX4, 0, ANY>;
     k.pass[3] = k.pass[6] = (const void *)&ntt_pass_kernel<F, 256, 3, RADIX4, 0, ANY>;
-    k.pass[5] = (const void *)&ntt_pass_kernel<F, 256, 4, RADIX2, 0, ANY>;
+    k.pass[5] = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX2, 0, ANY>;
+    set_wide<F, 5>(k);
+    set_wide<F, 6>(k);
+    set_wide<F, 7>(k);
+    set_wide<F, 8>(k);
     set_fixed<F, 5>(k);
     set_fixed<F, 6>(k);
     set_fixed<F, 7>(k);

@@ -198,6 +198,31 @@ __device__ __forceinline__ OutRows out_rows(const PassArgs &a, uint32_t tile, ui
     return o;
 }
 
+// x times the factors of row d in column cc formed on the fly
+template <class F>
+__device__ __forceinline__ void otf_scale(uint32_t x[8], const PassArgs &a, uint32_t tile, uint32_t d,
+                                          uint32_t cc) {
+    const uint4 *p[4];
+    otf_factors(p, a, tile, d, cc);
+#pragma unroll 1
+    while (p[0]) {
+        Factor v;
+        ldg_factor(v, p[0]);
+        mul_factor<F>(x, x, v);
+        p[0] = p[1];
+        p[1] = p[2];
+        p[2] = p[3];
+        p[3] = nullptr;
+    }
+}
+
+// the factor at f of the output's table (an entry of the big one is read once: it
+// takes no place in L1)
+__device__ __forceinline__ void ldg_out_factor(Factor &v, const PassArgs &a, const uint4 *f) {
+    if (a.last) ldg_factor(v, f);
+    else ldg_factor_stream(v, f);
+}
+
 // The rows at units u0 ^ i, times their output factors, to global memory: a
 // loop with one product in the code (unrolled, the kernels outgrow the
 // instruction cache).  The table's factor of the next row is read into the
@@ -236,20 +261,9 @@ __device__ __forceinline__ void scale_and_store(const PassArgs &a, const uint4 *
     }
 #pragma unroll 1
     for (uint32_t i = 0; i < R; i++) {
-        const uint4 *p[4];
-        otf_factors(p, a, tile, d0 + i, cc);
         uint32_t x[8];
         lds_elem(x, buf, u0 ^ i);
-#pragma unroll 1
-        while (p[0]) {
-            Factor v;
-            ldg_factor(v, p[0]);
-            mul_factor<F>(x, x, v);
-            p[0] = p[1];
-            p[1] = p[2];
-            p[2] = p[3];
-            p[3] = nullptr;
-        }
+        otf_scale<F>(x, a, tile, d0 + i, cc);
         st_elem8(o.out + 2 * i * o.step, x);
     }
 }
@@ -404,11 +418,67 @@ __device__ __forceinline__ void radix2_stage(uint4 *buf, const uint4 *tab, uint3
     }
 }
 
+// The stages of a tile one by one, one butterfly a thread and stage, and its
+// output: for transforms with few warps in flight, whose time is the chain of
+// products of one thread.  A digit of K bits is a chain of K - 1 products and two
+// independent ones for the output factors, where the radix-4 steps make up to
+// 2 K + 1 (2^12, digits 6 and 6: 12.4 -> 9.9 us, 2^14 14.4 -> 12.2, 2^15 16.4 ->
+// 14.4; 2^16, with a warp for every scheduler of the GPU, 17.2 -> 20.5).  EARLY: read the output
+// factors before the stages (32 registers held across them).
+template <class F, bool EARLY>
+__device__ __forceinline__ void run_stages(const PassArgs &a, const uint4 *tab, uint4 *buf,
+                                           uint32_t tile, uint32_t nthreads) {
+    const uint32_t K = a.K, lc = a.log_cols, tid = threadIdx.x;
+    const uint32_t half = 1u << (K + lc - 1);  // pairs in the tile
+    Factor v0, v1;
+    if (EARLY && tid < nthreads) {
+        const OutRows o = out_rows<2>(a, tile, (tid >> lc) << 1, tid & ((1u << lc) - 1u));
+        if (o.f) {
+            ldg_out_factor(v0, a, o.f);
+            ldg_out_factor(v1, a, o.f + o.fstep);
+        }
+    }
+    for (uint32_t h = 1u << (K - 1); h >= 2; h >>= 1) {
+        radix2_stage<F>(buf, tab, h, K, lc, tid, nthreads);
+        // at h <= 32 a warp's pairs, 32 consecutive ones, are made of rows of its
+        // own, at this stage and the next; the last (columns fastest) reads others'
+        if (h > 32 || h == 2) __syncthreads();
+        else __syncwarp();
+    }
+#pragma unroll 1
+    for (uint32_t g = tid; tid < nthreads && g < half; g += nthreads) {
+        const uint32_t cc = g & ((1u << lc) - 1u), d0 = (g >> lc) << 1;
+        const uint32_t u0 = smem_unit(cc, d0, K, lc);
+        const OutRows o = out_rows<2>(a, tile, d0, cc);
+        uint32_t x0[8], x1[8];
+        lds_elem(x0, buf, u0);
+        lds_elem(x1, buf, u0 ^ 1u);
+        sum_sub<F>(x0, x1);
+        if (o.f) {
+            if (!EARLY) ldg_out_factor(v0, a, o.f);
+            mul_factor<F>(x0, x0, v0);
+            if (!EARLY) ldg_out_factor(v1, a, o.f + o.fstep);
+            mul_factor<F>(x1, x1, v1);
+        } else if (!a.last) {
+            otf_scale<F>(x0, a, tile, d0, cc);
+            otf_scale<F>(x1, a, tile, d0 + 1, cc);
+        }
+        if (a.last) {
+            reduce_once<F>(x0);
+            reduce_once<F>(x1);
+        }
+        st_elem8(o.out, x0);
+        st_elem8(o.out + 2 * o.step, x1);
+    }
+}
+
 // Process one tile, copied to `buf` with the table in `tab` (the block has
 // synchronised since), with `nthreads` threads of the block (threads at or
 // beyond nthreads only take part in the barriers).  The block does not
 // synchronise at the end: `buf` may be written again after a barrier.
-template <class F, Steps STEPS>
+// EARLY: in the radix-2 form, whether the output factors are read before the stages
+// (a thread has one pair of each stage).
+template <class F, Steps STEPS, bool EARLY = false>
 __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, uint4 *buf,
                                          uint32_t tile, uint32_t nthreads) {
     const uint32_t K = a.K, lc = a.log_cols;
@@ -446,21 +516,21 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
         __syncthreads();
     }
 
+    if (STEPS == RADIX2 || (STEPS == EITHER && nthreads > (CN >> 2))) {
+        run_stages<F, EARLY>(a, tab, buf, tile, nthreads);
+        return;
+    }
+
     // the thread's entries of the big table are wanted in the last step: into L2
-    const uint32_t cc_out = tid & (C - 1), d_out = (tid >> lc) << 2;
+    // (by single prefetches: the bulk form takes one lane at a time)
     if (K >= 2 && !a.last && !a.otf && active && tid < (CN >> 2)) {
-        const OutRows o = out_rows<4>(a, tile, d_out, cc_out);
+        const OutRows o = out_rows<4>(a, tile, (tid >> lc) << 2, tid & (C - 1));
 #pragma unroll
         for (int i = 0; i < 4; i++) prefetch_l2(o.f + i * o.fstep);
     }
 
     // ---- stages 0 .. K-3
-    if (STEPS == RADIX2 || (STEPS == EITHER && nthreads > (CN >> 2))) {
-        for (uint32_t h = N >> 1; h >= 4; h >>= 1) {
-            radix2_stage<F>(buf, tab, h, K, lc, tid, nthreads);
-            __syncthreads();
-        }
-    } else if (K > 2) {
+    if (K > 2) {
         uint32_t q = N >> 2;  // distance of a radix-4 step's rows
         if (K & 1u) {
             radix2_stage<F>(buf, tab, N >> 1, K, lc, tid, nthreads);
@@ -638,7 +708,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) ntt_pass_kernel(const PassArg
     for (uint32_t fetch = blockIdx.x;; fetch += gridDim.x) {
         if (fetch < a.num_tiles) issue_tile_load(a, other, fetch, nthreads);
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (tile < a.num_tiles) run_tile<F, STEPS>(a, tab, cur, tile, nthreads);
+        if (tile < a.num_tiles) run_tile<F, STEPS, KIND != ANY>(a, tab, cur, tile, nthreads);
         if (fetch >= a.num_tiles) break;
         cp_async_wait_all();
         // the fetched tile is there, and every thread is done with the other one

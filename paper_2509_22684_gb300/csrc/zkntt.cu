@@ -302,11 +302,12 @@ zkntt_status device_info(DeviceInfo **out) {
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               PASS_MAX_SMEM));
         for (int f = 0; f < NUM_FIELDS; f++)
-            for (const auto &by_kind : field_kernels(f).fixed)
-                for (const void *k : by_kind)
-                    if (k)
-                        ZK_CHECK(cudaFuncSetAttribute(
-                            k, cudaFuncAttributeMaxDynamicSharedMemorySize, PASS_MAX_SMEM));
+            for (const auto &table : {field_kernels(f).fixed, field_kernels(f).wide})
+                for (int d = 0; d <= MAX_DIGIT_BITS; d++)
+                    for (const void *k : table[d])
+                        if (k)
+                            ZK_CHECK(cudaFuncSetAttribute(
+                                k, cudaFuncAttributeMaxDynamicSharedMemorySize, PASS_MAX_SMEM));
         for (int f = 0; f < NUM_FIELDS; f++) {
             ZK_CHECK(cudaFuncSetAttribute(batch_kernel_ptr(f),
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -524,10 +525,10 @@ zkntt_status split_tables(zkntt_plan_s *P, const HostField &F, const E8 &base, i
 // the variant's kernel of runtime sizes.
 zkntt_status set_launch(const PassPlan *ps, PassLaunch *r, int field, Kind kind, int sms) {
     const FieldKernels &kk = field_kernels(field);
-    const void *fixed = kk.fixed[ps->K][kind];
-    if (ps->ilp != 5 && ps->log_cols == fixed_cols(ps->K) && fixed) {
+    const void *fixed = (ps->ilp == 5 ? kk.wide : kk.fixed)[ps->K][kind];
+    if (ps->log_cols == fixed_cols(ps->K) && fixed) {
         r->kernel = fixed;
-        r->threads = 1 << (ps->K + ps->log_cols - 2);
+        r->threads = 1 << (ps->K + ps->log_cols - (ps->ilp == 5 ? 1 : 2));
     } else {
         r->kernel = kk.pass[ps->ilp];
         r->threads = int(pass_threads_for(uint32_t(ps->K), uint32_t(ps->log_cols), ps->ilp));
