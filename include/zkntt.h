@@ -241,15 +241,17 @@ zkntt_status zkntt_flags_destroy(uint32_t *host_view);
  *   d_h = cosetINTT_g(H)
  * with g the field's multiplicative generator.  d_a, d_b, d_c, d_h: n elements
  * each (inputs are read only; d_h must not overlap them).  d_scratch: 3 * n * 32
- * bytes of caller-owned device memory.  Runs the whole sequence as one
- * persistent launch (pointwise fused into the last transform's first pass);
- * further scratch comes from the library's stream-ordered pool.  log_n 1..28.
+ * bytes of caller-owned device memory.  Runs the sequence fused: the three
+ * independent transforms of a step share the launches of their passes, every
+ * launch follows the one before as its dependent, and the pointwise step is part
+ * of the last transform's first pass; further scratch (3 vectors) comes from the
+ * library's stream-ordered pool.  log_n 1..28.
  */
 zkntt_status zkntt_groth16_h(zkntt_field field, int log_n, const void *d_a, const void *d_b,
                              const void *d_c, void *d_h, void *d_scratch, void *stream);
 
-/* As zkntt_groth16_h (Fig. 2), choosing the form: fused = 1 is the single
- * persistent launch; fused = 0 issues the seven transforms and the pointwise
+/* As zkntt_groth16_h (Fig. 2), choosing the form: fused = 1 is the fused
+ * sequence; fused = 0 issues the seven transforms and the pointwise
  * kernel as separate launches (the form the paper finds in provers, Section
  * IV-A), for comparison. */
 zkntt_status zkntt_groth16_h_ex(zkntt_field field, int log_n, const void *d_a, const void *d_b,
@@ -259,7 +261,7 @@ zkntt_status zkntt_groth16_h_ex(zkntt_field field, int log_n, const void *d_a, c
 /*
  * The fused Groth16 H sequence (Fig. 2) captured once into a CUDA graph (the
  * launch-overhead reduction Section V-A points to): the capture
- * records the persistent launch and its stream-ordered scratch allocations
+ * records the launches and their stream-ordered scratch allocation
  * for these exact buffers; each zkntt_graph_launch replays it on `stream`
  * with no host-side work per transform.  `stream` must be a created stream
  * (not NULL) and idle during the call; the first call for a (field, log_n)

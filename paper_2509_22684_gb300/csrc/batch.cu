@@ -47,12 +47,10 @@ __global__ void __launch_bounds__(BATCH_THREADS, BATCH_MIN_BLOCKS)
                 }
                 segi = lo;
                 const BatchSeg &sg = tab.seg[segi];
-                for (int k = 0; k < 3 && !stop; k++) {
-                    if (sg.dep[k] < 0) continue;
-                    const uint32_t *cnt = done + sg.dep[k];
-                    if (ld_acquire(cnt) >= sg.dep_tiles[k]) continue;
+                const uint32_t *cnt = done + sg.dep;
+                if (sg.dep >= 0 && ld_acquire(cnt) < sg.dep_tiles) {
                     const unsigned long long t0 = global_ns();
-                    while (ld_acquire(cnt) < sg.dep_tiles[k]) {
+                    while (ld_acquire(cnt) < sg.dep_tiles) {
                         if (*(volatile uint32_t *)&ctrl[1]) { stop = 1; break; }
                         if (global_ns() - t0 > tab.timeout_ns) {
                             atomicExch(&ctrl[1], 1u);

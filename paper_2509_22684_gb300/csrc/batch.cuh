@@ -1,18 +1,17 @@
-// batch.cuh -- persistent kernel running many transforms (uneven sizes, with
-// dependencies between them) in one launch per field.
+// batch.cuh -- persistent kernel running many independent transforms of uneven
+// sizes in one launch per field.
 //
-// The paper finds that the Groth16 prover runs seven transforms, every one of
-// them as several kernel launches (Section IV-A), and that such short kernels run
-// with sub-optimal launch parameters; it calls for runtime autotuning (Section
-// V-A).  Here every pass of every transform is a segment of tiles; all tiles of
-// all segments form one work list ordered by dependency level.  Resident
-// blocks (one grid sized to the SM count) pull the next tile index from a
-// device counter.  A segment may depend on up to three earlier segments (the
-// previous pass of the same transform, or the producers of its input); the
-// block that claims a tile waits until those segments have retired all their
-// tiles.  Because tiles are claimed in list order and every dependency points
-// to an earlier position, the oldest unfinished tile can always run, so the
-// scheme cannot deadlock however many blocks are resident.
+// The paper finds that short kernels run with sub-optimal launch parameters and
+// calls for runtime autotuning (Section V-A); a server's batch holds many
+// transforms too small to fill the GPU.  Here every pass of every transform is a
+// segment of tiles; all tiles of all segments form one work list ordered by
+// dependency level.  Resident blocks (one grid sized to the SM count) pull the
+// next tile index from a device counter.  A segment may depend on an earlier one,
+// the previous pass of the same transform; the block that claims a tile waits
+// until that segment has retired all its tiles.  Because tiles are claimed in list
+// order and every dependency points to an earlier position, the oldest unfinished
+// tile can always run, so the scheme cannot deadlock however many blocks are
+// resident.
 //
 // Every wait is bounded by `timeout_ns` (device global timer).  On expiry the
 // block sets the launch's abort word and the sticky status word, and all blocks
@@ -42,8 +41,8 @@ struct BatchSeg {
     PassArgs a;
     uint32_t K;           // digit bits of this pass
     uint32_t first_item;  // index of the segment's first tile in the work list
-    int32_t dep[3];       // segments that must be complete first (-1: none)
-    uint32_t dep_tiles[3];
+    int32_t dep;          // segment that must be complete first (-1: none)
+    uint32_t dep_tiles;   // its tiles
     uint32_t ntiles;      // tiles in this segment
     uint32_t job;         // index of the transform in the batch
     uint32_t signal;      // 1: last pass of its transform and completion words requested

@@ -78,6 +78,21 @@ struct PassArgs {
     uint32_t num_tiles;   // tiles in this pass
 };
 
+// The vectors of a launch: up to three of one plan, whose tiles follow each other
+// (three independent transforms fill the GPU where one does not).
+constexpr int PASS_VECTORS = 3;
+struct PassVectors {
+    const uint4 *in[PASS_VECTORS];
+    uint4 *out[PASS_VECTORS];
+    uint32_t tiles;  // tiles of one vector
+};
+
+// the tile within its vector v
+__device__ __forceinline__ uint32_t vector_tile(const PassVectors &vec, uint32_t tile, uint32_t &v) {
+    for (v = 0; tile >= vec.tiles; v++) tile -= vec.tiles;
+    return tile;
+}
+
 __device__ __forceinline__ uint32_t brev_bits(uint32_t x, uint32_t bits) {
     return bits == 0 ? 0u : (__brev(x) >> (32 - bits));
 }
@@ -684,9 +699,12 @@ __device__ __forceinline__ void fix_args(PassArgs &a) {
     if (KIND != LAST_POST) a.post = nullptr;
 }
 
-// One pass.  The register budget is for BLOCKS blocks of THREADS threads an SM.
+// One pass over the vectors' tiles (args: num_tiles of them in all; its own `in`
+// and `out` are not used).  The register budget is for BLOCKS blocks of THREADS
+// threads an SM.
 template <class F, int THREADS, int BLOCKS, Steps STEPS, int K, Kind KIND>
-__global__ void __launch_bounds__(THREADS, BLOCKS) ntt_pass_kernel(const PassArgs args) {
+__global__ void __launch_bounds__(THREADS, BLOCKS)
+    ntt_pass_kernel(const PassArgs args, const __grid_constant__ PassVectors vec) {
     extern __shared__ uint4 smem[];
     PassArgs a = args;
     fix_args<K, KIND>(a);
@@ -706,9 +724,19 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) ntt_pass_kernel(const PassArg
     uint4 *cur = buf + units, *other = buf;
 #pragma unroll 1
     for (uint32_t fetch = blockIdx.x;; fetch += gridDim.x) {
-        if (fetch < a.num_tiles) issue_tile_load(a, other, fetch, nthreads);
-        else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (tile < a.num_tiles) run_tile<F, STEPS, KIND != ANY>(a, tab, cur, tile, nthreads);
+        uint32_t v;
+        if (fetch < a.num_tiles) {
+            const uint32_t t = vector_tile(vec, fetch, v);
+            a.in = vec.in[v];
+            issue_tile_load(a, other, t, nthreads);
+        } else {
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        }
+        if (tile < a.num_tiles) {
+            const uint32_t t = vector_tile(vec, tile, v);
+            a.out = vec.out[v];
+            run_tile<F, STEPS, KIND != ANY>(a, tab, cur, t, nthreads);
+        }
         if (fetch >= a.num_tiles) break;
         cp_async_wait_all();
         // the fetched tile is there, and every thread is done with the other one

@@ -376,8 +376,9 @@ zkntt_status pool_alloc(void **p, size_t bytes, cudaStream_t s) {
 // how a pass is launched
 struct PassLaunch {
     const void *kernel = nullptr;
-    int threads = 0, grid = 0;
-    size_t smem = 0;
+    int threads = 0;
+    size_t smem[2] = {};     // with one and with two tile buffers
+    uint32_t slots[2] = {};  // blocks that fit the GPU so
 };
 
 struct PassPlan {
@@ -533,17 +534,16 @@ zkntt_status set_launch(const PassPlan *ps, PassLaunch *r, int field, Kind kind,
         r->kernel = kk.pass[ps->ilp];
         r->threads = int(pass_threads_for(uint32_t(ps->K), uint32_t(ps->log_cols), ps->ilp));
     }
-    // the twiddle table and the tile buffers: one will do if every block has one tile
+    // the twiddle table and the tile buffers
     const size_t tile_bytes = size_t(16) * tile_units(1u << (ps->K + ps->log_cols));
     const size_t table_bytes = size_t(64) * tab_entries(uint32_t(ps->K));
-    int nb = 0;
-    for (int n = 1; n <= 2; n++) {
-        r->smem = table_bytes + n * tile_bytes;
-        ZK_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, r->kernel, r->threads, r->smem));
-        nb = std::max(nb, 1);
-        if (ps->num_tiles <= uint64_t(nb) * sms) break;
+    for (int n = 0; n < 2; n++) {
+        int nb = 0;
+        r->smem[n] = table_bytes + (n + 1) * tile_bytes;
+        ZK_CHECK(
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, r->kernel, r->threads, r->smem[n]));
+        r->slots[n] = uint32_t(std::max(nb, 1)) * uint32_t(sms);
     }
-    r->grid = int(std::min<uint64_t>(ps->num_tiles, uint64_t(nb) * sms));
     return ZKNTT_OK;
 }
 
@@ -803,41 +803,53 @@ zkntt_status check_plan_device(const zkntt_plan_s *P) {
     return cur == P->device ? ZKNTT_OK : ZKNTT_EINVAL;
 }
 
-// pw_b, pw_c (both or neither): the transform of in * pw_b - pw_c
-zkntt_status run_passes(const zkntt_plan_s *P, const void *in, void *out, void *scratch,
-                        cudaStream_t s, const void *pw_b = nullptr, const void *pw_c = nullptr) {
+// `count` transforms of one plan, in[k] -> out[k] through scratch[k], pass by pass.
+// pw_b, pw_c (both or neither, for one transform): of in * pw_b - pw_c.
+// follows: the work before it on the stream is this function's too.
+zkntt_status run_passes(const zkntt_plan_s *P, int count, const void *const *in, void *const *out,
+                        void *const *scratch, cudaStream_t s, const void *pw_b = nullptr,
+                        const void *pw_c = nullptr, bool follows = false) {
     for (int i = 0; i < P->passes; i++) {
-        const void *src = (i == 0) ? in : scratch;
-        void *dst = (i == P->passes - 1) ? out : scratch;
-        PassArgs a = pass_args(P, i, src, dst);
+        PassArgs a = pass_args(P, i, nullptr, nullptr);
+        PassVectors vec;
+        memset(&vec, 0, sizeof vec);
+        vec.tiles = a.num_tiles;
+        a.num_tiles *= uint32_t(count);
+        for (int k = 0; k < count; k++) {
+            vec.in[k] = static_cast<const uint4 *>(i == 0 ? in[k] : scratch[k]);
+            vec.out[k] = static_cast<uint4 *>(i == P->passes - 1 ? out[k] : scratch[k]);
+        }
         if (i == 0) {
             a.pw_b = static_cast<const uint4 *>(pw_b);
             a.pw_c = static_cast<const uint4 *>(pw_c);
         }
-        void *args[] = {&a};
+        void *args[] = {&a, &vec};
         const PassLaunch &r = (i == 0 && pw_b) ? P->ps[i].run_pw : P->ps[i].run;
-        if (i == 0) {
-            // the first pass is ordered after all earlier work on the stream
-            // (which may write `in`)
-            ZK_CHECK(cudaLaunchKernel(r.kernel, dim3(r.grid), dim3(r.threads), args, r.smem, s));
-            continue;
-        }
-        // later passes depend only on the pass before: a programmatic
-        // dependent launch overlaps their launch with its tail (the kernel
-        // waits for the previous pass's completion before any memory access)
+        // one tile buffer will do if every block has one tile
+        const int two = a.num_tiles > r.slots[0];
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(r.grid);
+        cfg.gridDim = dim3(std::min(a.num_tiles, r.slots[two]));
         cfg.blockDim = dim3(r.threads);
-        cfg.dynamicSmemBytes = r.smem;
+        cfg.dynamicSmemBytes = r.smem[two];
         cfg.stream = s;
+        // A first pass is ordered after all earlier work on the stream (which may
+        // write `in`).  Later passes, and the first of a transform that follows
+        // another here, depend only on the pass before: a programmatic dependent
+        // launch overlaps their launch with its tail (every pass kernel waits for
+        // the one before to complete before any access to the vectors).
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = i > 0 || follows;
         ZK_CHECK(cudaLaunchKernelExC(&cfg, r.kernel, args));
     }
     return ZKNTT_OK;
+}
+
+zkntt_status run_passes(const zkntt_plan_s *P, const void *in, void *out, void *scratch,
+                        cudaStream_t s) {
+    return run_passes(P, 1, &in, &out, &scratch, s);
 }
 
 // Scratch for zkntt_execute_noalloc: a file-scope device array, so that entry
@@ -912,9 +924,7 @@ struct JobSpec {
     const void *in;
     void *out;
     void *scratch;
-    const void *pw_b = nullptr, *pw_c = nullptr;  // fused pointwise on the first pass
-    int level0 = 0;                               // level of the job's first pass
-    int deps[3] = {-1, -1, -1};                   // jobs whose last pass must finish first
+    int level0 = 0;  // level of the job's first pass
 };
 
 // One persistent launch over jobs of one field (job_ids: completion-word index
@@ -975,38 +985,20 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
         sg.a = pass_args(P, i, src, dst);
         sg.a.log_cols = uint32_t(batch_log_cols(P, i));
         sg.a.num_tiles = batch_tiles(P, i);
-        if (i == 0) {
-            sg.a.pw_b = static_cast<const uint4 *>(J.pw_b);
-            sg.a.pw_c = static_cast<const uint4 *>(J.pw_c);
-        }
         sg.K = uint32_t(P->ps[i].K);
         sg.first_item = item;
         sg.ntiles = sg.a.num_tiles;
         sg.job = job_ids[segs[k].job];
         sg.signal = (flags && i == P->passes - 1) ? 1u : 0u;
         item += sg.a.num_tiles;
-        for (int d = 0; d < 3; d++) {
-            sg.dep[d] = -1;
-            sg.dep_tiles[d] = 0;
-        }
+        // the pass before: an earlier segment of the work list (its level is lower),
+        // which is what makes the persistent schedule deadlock-free
+        sg.dep = -1;
+        sg.dep_tiles = 0;
         if (i > 0) {
-            int dk = index[{segs[k].job, i - 1}];
-            sg.dep[0] = dk;
-            sg.dep_tiles[0] = batch_tiles(jobs[segs[k].job].plan, i - 1);
-        } else {
-            for (int d = 0; d < 3; d++) {
-                int dj = J.deps[d];
-                if (dj < 0) continue;
-                const zkntt_plan_s *DP = jobs[dj].plan;
-                int dk = index[{dj, DP->passes - 1}];
-                sg.dep[d] = dk;
-                sg.dep_tiles[d] = batch_tiles(DP, DP->passes - 1);
-            }
-        }
-        // every dependency must point to an earlier segment of the work list:
-        // that ordering is what makes the persistent schedule deadlock-free
-        for (int d = 0; d < 3; d++) {
-            if (sg.dep[d] >= k) {
+            sg.dep = index[{segs[k].job, i - 1}];
+            sg.dep_tiles = batch_tiles(P, i - 1);
+            if (sg.dep >= k) {
                 delete tab;
                 return ZKNTT_EINVAL;
             }
@@ -1064,7 +1056,7 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
 }
 
 // Jobs of several fields run as one persistent launch per field, in order of
-// each field's first job, on stream s (a dependency must stay within a field).
+// each field's first job, on stream s.
 zkntt_status launch_batch(const std::vector<JobSpec> &jobs, cudaStream_t s,
                           unsigned long long timeout_ns, uint32_t *flags = nullptr,
                           uint32_t epoch = 0, const std::vector<uint32_t> *job_ids = nullptr) {
@@ -1075,19 +1067,11 @@ zkntt_status launch_batch(const std::vector<JobSpec> &jobs, cudaStream_t s,
     for (int f : order) {
         std::vector<JobSpec> sub;
         std::vector<uint32_t> ids;
-        std::vector<int> local(jobs.size(), -1);
         for (int j = 0; j < int(jobs.size()); j++) {
             if (jobs[j].plan->field != f) continue;
-            local[j] = int(sub.size());
             sub.push_back(jobs[j]);
             ids.push_back(job_ids ? (*job_ids)[j] : uint32_t(j));
         }
-        for (JobSpec &J : sub)
-            for (int d = 0; d < 3; d++) {
-                if (J.deps[d] < 0) continue;
-                if (local[J.deps[d]] < 0) return ZKNTT_EINVAL;  // dependency across fields
-                J.deps[d] = local[J.deps[d]];
-            }
         zkntt_status st = launch_batch_field(sub, s, timeout_ns, flags, epoch, ids);
         if (st != ZKNTT_OK) return st;
     }
@@ -1100,13 +1084,6 @@ unsigned long long batch_timeout_ns() {
     if (ms == 0) ms = 2000;
     return ms * 1000000ull;
 }
-
-// From this size on the fused Groth16 sequence runs its transforms one after the
-// other as passes of the compiled kernels (each fills the GPU), below it as one
-// persistent launch, whose three independent transforms share the GPU.  Graph
-// replays, BLS12-381, persistent / passes: 2^16 109 / 117 us, 2^17 201 / 175,
-// 2^18 338 / 318, 2^20 1129 / 1189, 2^21 2536 / 2353, 2^22 5204 / 4745.
-constexpr int G16_PASSES_LOG_N = 17;
 
 // Groth16 plans per (field, log_n).  Separate form (the sequence as stated):
 // iNTT, coset NTT, coset iNTT.  Fused form: cosetNTT_g(iNTT(a)) is computed as
@@ -1443,53 +1420,17 @@ zkntt_status zkntt_groth16_h_ex(zkntt_field field, int log_n, const void *d_a, c
         if (st2 != ZKNTT_OK) return st2;
         return zkntt_execute(G->cintt, d_h, d_h, s);
     }
-    if (log_n >= G16_PASSES_LOG_N) {
-        const size_t need = scratch_bytes_of(G->ntt);
-        void *ps = nullptr;
-        if (need && (st = pool_alloc(&ps, need, s))) return st;
-        for (int k = 0; k < 3 && st == ZKNTT_OK; k++) st = run_passes(G->intt_gj, in[k], sv[k], ps, s);
-        for (int k = 0; k < 3 && st == ZKNTT_OK; k++) st = run_passes(G->ntt, sv[k], sv[k], ps, s);
-        if (st == ZKNTT_OK) st = run_passes(G->cintt_z, S0, d_h, ps, s, S1, S2);
-        if (ps) {
-            zkntt_status st2 = from_cuda(cudaFreeAsync(ps, s));
-            if (st == ZKNTT_OK) st = st2;
-        }
-        return st;
-    }
-    // fused: one persistent launch over the dependency graph
-    //   jobs 0-2: cosetINTT_{g^-1}(a|b|c) -> S0|S1|S2   levels 0 .. p-1
-    //   jobs 3-5: NTT in place on S0|S1|S2              levels p .. 2p-1
-    //   job 6:    cosetINTT_g(S0*S1 - S2) * zinv -> h   levels 2p .. 3p-1
-    const size_t per = scratch_bytes_of(G->ntt);
+    // fused: cosetINTT_{g^-1}(a, b, c) -> S0, S1, S2 and NTT in place on them, three
+    // transforms a launch, then cosetINTT_g(S0 S1 - S2) zinv -> h
+    const size_t per = std::max({scratch_bytes_of(G->intt_gj), scratch_bytes_of(G->ntt),
+                                 scratch_bytes_of(G->cintt_z)});
     char *ps = nullptr;
-    if (per) {
-        zkntt_status sa = pool_alloc(reinterpret_cast<void **>(&ps), 7 * per, s);
-        if (sa != ZKNTT_OK) return sa;
-    }
-    std::vector<JobSpec> jobs(7);
-    const int p1 = G->intt_gj->passes, p2 = G->ntt->passes;
-    for (int k = 0; k < 3; k++) {
-        jobs[k].plan = G->intt_gj;
-        jobs[k].in = in[k];
-        jobs[k].out = sv[k];
-        jobs[k].level0 = 0;
-        jobs[3 + k].plan = G->ntt;
-        jobs[3 + k].in = sv[k];
-        jobs[3 + k].out = sv[k];
-        jobs[3 + k].level0 = p1;
-        jobs[3 + k].deps[0] = k;
-    }
-    jobs[6].plan = G->cintt_z;
-    jobs[6].in = S0;
-    jobs[6].out = d_h;
-    jobs[6].pw_b = S1;
-    jobs[6].pw_c = S2;
-    jobs[6].level0 = p1 + p2;
-    jobs[6].deps[0] = 3;
-    jobs[6].deps[1] = 4;
-    jobs[6].deps[2] = 5;
-    for (int j = 0; j < 7; j++) jobs[j].scratch = per ? ps + j * per : nullptr;
-    st = launch_batch(jobs, s, batch_timeout_ns());
+    if (per && (st = pool_alloc(reinterpret_cast<void **>(&ps), 3 * per, s))) return st;
+    void *const scr[3] = {ps, per ? ps + per : nullptr, per ? ps + 2 * per : nullptr};
+    const void *const sin[3] = {S0, S1, S2};
+    st = run_passes(G->intt_gj, 3, in, sv, scr, s);
+    if (st == ZKNTT_OK) st = run_passes(G->ntt, 3, sin, sv, scr, s, nullptr, nullptr, true);
+    if (st == ZKNTT_OK) st = run_passes(G->cintt_z, 1, sin, &d_h, scr, s, S1, S2, true);
     if (ps) {
         zkntt_status st2 = from_cuda(cudaFreeAsync(ps, s));
         if (st == ZKNTT_OK) st = st2;
@@ -1601,9 +1542,8 @@ zkntt_status zkntt_inject_timeout(int timeout_ms, void *stream) {
     tab->timeout_ns = (unsigned long long)timeout_ms * 1000000ull;
     tab->seg[0].K = 4;
     tab->seg[0].first_item = 0;
-    tab->seg[0].dep[0] = 0;
-    tab->seg[0].dep[1] = tab->seg[0].dep[2] = -1;
-    tab->seg[0].dep_tiles[0] = 1;
+    tab->seg[0].dep = 0;
+    tab->seg[0].dep_tiles = 1;
     uint32_t *ctrl = nullptr;
     st = pool_alloc(reinterpret_cast<void **>(&ctrl), 3 * 4, s);
     if (st != ZKNTT_OK) {
