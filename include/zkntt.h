@@ -78,11 +78,9 @@ typedef struct {
     int use_tuner;         /* 0 or 1: use a tuned schedule when one is known for this GPU
                               (zkntt_tuned.jsonl beside the library, then ZKNTT_TUNE_CACHE);
                               -1: never (planner heuristic only) */
-    int ilp;               /* kernel variant: two stages at a time, four elements a thread, with
-                              registers for 5 blocks of 128 threads per SM (1 and 7) or for
-                              2 (2 and 4) or 3 (3 and 6) blocks of 256; 5 = one butterfly
-                              per thread per stage, registers for 2 blocks of 256 (for
-                              small transforms); 0 = auto; outside 0..7 -> ZKNTT_EINVAL */
+    int ilp;               /* kernel variant: 1..4, 6, 7 = two stages at a time, four elements a
+                              thread; 5 = one butterfly per thread per stage (for small
+                              transforms); 0 = auto; outside 0..7 -> ZKNTT_EINVAL */
 } zkntt_plan_options;
 
 /*

@@ -152,22 +152,35 @@ __global__ void field_op_kernel(int op, const uint4 *a, const uint4 *b, uint4 *c
     }
 }
 
-// Groth16 pointwise on the coset: h = (a * b - c) * z
+// Groth16 pointwise on the coset: h = (a * b - c) * z.  Bound by its two products
+// (75 us of Montgomery products at 3 million elements, 57 us of memory): z is a
+// constant, so the second is a factor's, with the factor in the kernel's
+// parameters; the next element's vectors are read while this one's products run,
+// into the registers that are done with.  3,000,001 elements: 89 -> 82 us.
 template <class F>
-__global__ void pointwise_kernel(const uint4 *a, const uint4 *b, const uint4 *c, const uint4 *z,
-                                 uint4 *h, size_t n) {
-    uint32_t zz[8];
-    ldg_elem(zz, z);
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += size_t(gridDim.x) * blockDim.x) {
-        uint32_t x[8], y[8], w[8];
-        ldg_elem(x, a + 2 * i);
-        ldg_elem(y, b + 2 * i);
-        mul<F>(x, x, y);
-        ldg_elem(w, c + 2 * i);
-        sub<F>(x, x, w);
-        mul<F>(x, x, zz);
-        st_elem(h + 2 * i, x);
+__global__ void __launch_bounds__(128, 5)
+    pointwise_kernel(const uint4 *a, const uint4 *b, const uint4 *c,
+                     const __grid_constant__ Factor z, uint4 *h, size_t n) {
+    const size_t step = size_t(gridDim.x) * blockDim.x;
+    size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint32_t x[8], y[8], w[8], v[8];
+    ldg_elem(x, a + 2 * i);
+    ldg_elem(y, b + 2 * i);
+    ldg_elem(w, c + 2 * i);
+#pragma unroll 1
+    for (;; i += step) {
+        const bool more = n - i > step;
+        const size_t k = more ? i + step : i;
+        mul<F>(v, x, y);
+        ldg_elem(x, a + 2 * k);
+        ldg_elem(y, b + 2 * k);
+        sub<F>(v, v, w);
+        ldg_elem(w, c + 2 * k);
+        mul_factor<F>(v, v, z);
+        reduce_once<F>(v);
+        st_elem8(h + 2 * i, v);
+        if (!more) break;
     }
 }
 

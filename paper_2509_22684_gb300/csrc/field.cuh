@@ -189,33 +189,31 @@ __device__ __forceinline__ void add_loose(uint32_t r[8], const uint32_t a[8], co
 template <class F>
 __device__ __forceinline__ void sub_loose(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
     using D = Twice<F>;
-    uint32_t mask, u[8];
-    asm("sub.cc.u32  %0, %9, %17;\n\t"
-        "subc.cc.u32 %1, %10, %18;\n\t"
-        "subc.cc.u32 %2, %11, %19;\n\t"
-        "subc.cc.u32 %3, %12, %20;\n\t"
-        "subc.cc.u32 %4, %13, %21;\n\t"
-        "subc.cc.u32 %5, %14, %22;\n\t"
-        "subc.cc.u32 %6, %15, %23;\n\t"
-        "subc.cc.u32 %7, %16, %24;\n\t"
-        "subc.u32    %8, 0, 0;"
-        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
-          "=r"(u[7]), "=r"(mask)
+    asm("{\n\t.reg .pred p;\n\t.reg .u32 m;\n\t"
+        "sub.cc.u32  %0, %8, %16;\n\t"
+        "subc.cc.u32 %1, %9, %17;\n\t"
+        "subc.cc.u32 %2, %10, %18;\n\t"
+        "subc.cc.u32 %3, %11, %19;\n\t"
+        "subc.cc.u32 %4, %12, %20;\n\t"
+        "subc.cc.u32 %5, %13, %21;\n\t"
+        "subc.cc.u32 %6, %14, %22;\n\t"
+        "subc.cc.u32 %7, %15, %23;\n\t"
+        "subc.u32    m, 0, 0;\n\t"
+        "setp.ne.u32 p, m, 0;\n\t"
+        "@p add.cc.u32  %0, %0, %24;\n\t"
+        "@p addc.cc.u32 %1, %1, %25;\n\t"
+        "@p addc.cc.u32 %2, %2, %26;\n\t"
+        "@p addc.cc.u32 %3, %3, %27;\n\t"
+        "@p addc.cc.u32 %4, %4, %28;\n\t"
+        "@p addc.cc.u32 %5, %5, %29;\n\t"
+        "@p addc.cc.u32 %6, %6, %30;\n\t"
+        "@p addc.u32    %7, %7, %31;\n\t}"
+        : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]),
+          "=&r"(r[7])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
-          "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7]));
-    asm("add.cc.u32  %0, %8, %16;\n\t"
-        "addc.cc.u32 %1, %9, %17;\n\t"
-        "addc.cc.u32 %2, %10, %18;\n\t"
-        "addc.cc.u32 %3, %11, %19;\n\t"
-        "addc.cc.u32 %4, %12, %20;\n\t"
-        "addc.cc.u32 %5, %13, %21;\n\t"
-        "addc.cc.u32 %6, %14, %22;\n\t"
-        "addc.u32    %7, %15, %23;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7])
-        : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]),
-          "r"(D::D0 & mask), "r"(D::D1 & mask), "r"(D::D2 & mask), "r"(D::D3 & mask),
-          "r"(D::D4 & mask), "r"(D::D5 & mask), "r"(D::D6 & mask), "r"(D::D7 & mask));
+          "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7]),
+          "n"(D::D0), "n"(D::D1), "n"(D::D2), "n"(D::D3), "n"(D::D4), "n"(D::D5), "n"(D::D6),
+          "n"(D::D7));
 }
 
 // r congruent to a - b for loose a, b, only to be multiplied by a factor: where

@@ -8,11 +8,11 @@
 namespace zkntt {
 
 // the pass kernels compiled for a digit of K bits: one thread per four elements
-// of a tile, 96 registers (128 when that makes 256 threads)
+// of a tile, 128 registers (2^24: 2594 us, with 96 2606, with 80 2702)
 template <class F, int K, Kind KIND>
 const void *fixed_kernel() {
     constexpr int T = 1 << (K + fixed_cols(K) - 2);
-    constexpr int B = T >= 256 ? 2 : T >= 32 ? 640 / T : 20;
+    constexpr int B = T >= 32 ? 512 / T : 16;
     return (const void *)&ntt_pass_kernel<F, T, B, RADIX4, K, KIND>;
 }
 
@@ -43,11 +43,8 @@ void set_fixed(FieldKernels &k) {
 template <class F>
 FieldKernels make_field_kernels() {
     FieldKernels k = {};
-    // registers: 96 (variants 1 and 7), 128 (2, 4 and 5), 80 (3 and 6)
-    k.pass[1] = k.pass[7] = (const void *)&ntt_pass_kernel<F, 128, 5, RADIX4, 0, ANY>;
-    k.pass[2] = k.pass[4] = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX4, 0, ANY>;
-    k.pass[3] = k.pass[6] = (const void *)&ntt_pass_kernel<F, 256, 3, RADIX4, 0, ANY>;
-    k.pass[5] = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX2, 0, ANY>;
+    k.any4 = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX4, 0, ANY>;
+    k.any2 = (const void *)&ntt_pass_kernel<F, 256, 2, RADIX2, 0, ANY>;
     set_wide<F, 5>(k);
     set_wide<F, 6>(k);
     set_wide<F, 7>(k);

@@ -9,7 +9,7 @@ constexpr int MAX_DIGIT_BITS = 11;  // largest sub-transform a block holds (2^11
 constexpr int MAX_TILE_BITS = 11;   // tiles hold at most 2^11 elements (C x 2^K)
 
 struct FieldKernels {
-    const void *pass[8];  // the pass kernel of schedule variant 1..7 (digit size is a runtime argument)
+    const void *any4, *any2;  // the pass kernels of runtime sizes: radix 4, radix 2 (variant 5)
     const void *fixed[MAX_DIGIT_BITS + 1][6];  // pass kernels by digit bits and Kind (null: none)
     const void *wide[MAX_DIGIT_BITS + 1][6];   // the same with one thread per pair (variant 5)
     const void *gen_powers;

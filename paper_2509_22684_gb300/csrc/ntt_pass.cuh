@@ -243,8 +243,9 @@ __device__ __forceinline__ void ldg_out_factor(Factor &v, const PassArgs &a, con
 // instruction cache).  The table's factor of the next row is read into the
 // registers of the present one as soon as the product is done with them: its
 // quotient during the second half of the product, its value during the store and
-// the first half of the next.
-template <class F, int R>
+// the first half of the next.  AHEAD: factors on the fly too (the batch kernel, with
+// 80 registers, reads those when it needs them).
+template <class F, int R, bool AHEAD>
 __device__ __forceinline__ void scale_and_store(const PassArgs &a, const uint4 *buf, uint32_t u0,
                                                 const OutRows &o, uint32_t tile, uint32_t d0,
                                                 uint32_t cc) {
@@ -274,12 +275,49 @@ __device__ __forceinline__ void scale_and_store(const PassArgs &a, const uint4 *
         }
         return;
     }
+    if (!AHEAD) {
 #pragma unroll 1
-    for (uint32_t i = 0; i < R; i++) {
-        uint32_t x[8];
-        lds_elem(x, buf, u0 ^ i);
-        otf_scale<F>(x, a, tile, d0 + i, cc);
+        for (uint32_t i = 0; i < R; i++) {
+            uint32_t x[8];
+            lds_elem(x, buf, u0 ^ i);
+            otf_scale<F>(x, a, tile, d0 + i, cc);
+            st_elem8(o.out + 2 * i * o.step, x);
+        }
+        return;
+    }
+    // on the fly: the two to four factors of each row one after the other, read ahead
+    // in the same way (2^22, BN254: 783 -> 758 us)
+    const uint32_t lo_tiles_bits = a.lo_bits - a.log_cols;
+    const uint32_t lo = ((tile & ((1u << lo_tiles_bits) - 1u)) << a.log_cols) + cc;
+    // lo < 2^lo_bits and rev(d) < 2^K, so the exponent is below 2^tw_bits = n_i: no
+    // reduction (and no overflow: tw_bits <= 32); row i adds rev(i) parts of it
+    const uint32_t e0 = lo * brev_bits(d0, a.K), part = lo << (a.K - (R == 4 ? 2 : 1));
+    const uint32_t factors = 2 + (a.fl != nullptr) + (a.fd != nullptr);
+    auto factor = [&](uint32_t i, uint32_t j) -> const uint4 * {
+        const uint32_t e = e0 + part * (R == 4 ? ((i & 1u) << 1) | (i >> 1) : i);
+        if (j == 0) return a.w_hi + 4 * size_t(e >> a.split_bits);
+        if (j == 1) return a.w_lo + 4 * size_t(e & ((1u << a.split_bits) - 1u));
+        return j == 2 && a.fl ? a.fl + 4 * size_t(lo) : a.fd + 4 * size_t(d0 + i);
+    };
+    Factor v;
+    ldg_factor(v, factor(0, 0));
+    uint32_t x[8], q[8];
+    lds_elem(x, buf, u0);
+#pragma unroll 1
+    for (uint32_t i = 0, j = 0;;) {
+        mul_high(q, x, v.wq);
+        const bool row_done = j + 1 == factors, done = row_done && i + 1 == R;
+        const uint4 *f = done ? a.w_hi : row_done ? factor(i + 1, 0) : factor(i, j + 1);
+        ZK_LD8("", v.wq, f + 2);
+        mul_low_fold<F>(x, x, v.w, q);
+        ZK_LD8("", v.w, f);
+        j++;
+        if (!row_done) continue;
         st_elem8(o.out + 2 * i * o.step, x);
+        if (done) break;
+        i++;
+        j = 0;
+        lds_elem(x, buf, u0 ^ i);
     }
 }
 
@@ -386,10 +424,6 @@ __device__ __forceinline__ void lds_factor(Factor &f, const uint4 *tab, uint32_t
     lds_elem(f.wq, tab, u + 16);
 }
 
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 // How a tile's stages run: two at a time, four elements a thread (radix 4), or
 // one by one, one butterfly a thread (radix 2); or either by the thread count.
 enum Steps { RADIX4 = 1, RADIX2 = 2, EITHER = 3 };
@@ -409,6 +443,17 @@ __device__ __forceinline__ void sum_sub(uint32_t x[8], uint32_t y[8]) {
     add_loose<F>(x, x, y);
 #pragma unroll
     for (int k = 0; k < 8; k++) y[k] = t[k];
+}
+
+// two products side by side
+template <class F>
+__device__ __forceinline__ void mul_factor2(uint32_t r[8], const uint32_t x[8], const Factor &f,
+                                            uint32_t s[8], const uint32_t y[8], const Factor &g) {
+    uint32_t p[8], q[8];
+    mul_high(p, x, f.wq);
+    mul_high(q, y, g.wq);
+    mul_low_fold<F>(r, x, f.w, p);
+    mul_low_fold<F>(s, y, g.w, q);
 }
 
 // One stage, pairs at distance h, one butterfly after the other.
@@ -503,30 +548,57 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
     const uint32_t tid = threadIdx.x;
     const bool active = tid < nthreads;
 
-    // ---- input factors
-    if (a.pre || a.pw_b) {
+    // ---- input factors.  Each is read into the registers of the one before it as
+    // soon as that has been used (not in the batch kernel, with 80 registers and
+    // without the pointwise step).
+    auto place = [&](uint32_t e, uint32_t &d, uint32_t &cc) {
+        if (a.last) { d = e & (N - 1); cc = e >> K; }
+        else        { cc = e & (C - 1); d = e >> lc; }
+    };
+    if (STEPS == EITHER && a.pre) {
 #pragma unroll 1
         for (uint32_t e = tid; active && e < CN; e += nthreads) {
-            uint32_t d, cc;
-            if (a.last) { d = e & (N - 1); cc = e >> K; }
-            else        { cc = e & (C - 1); d = e >> lc; }
-            const uint32_t s = smem_unit(cc, d, K, lc);
-            uint32_t x[8];
-            lds_elem(x, buf, s);
+            uint32_t d, cc, x[8];
+            place(e, d, cc);
+            const uint32_t u = smem_unit(cc, d, K, lc);
+            Factor f;
+            ldg_factor(f, a.pre + 4 * size_t(d));
+            lds_elem(x, buf, u);
+            mul_factor<F>(x, x, f);
+            sts_elem(buf, u, x);
+        }
+        __syncthreads();
+    }
+    if (STEPS != EITHER && (a.pre || a.pw_b)) {
+        uint32_t d, cc, b[8], c[8];
+        Factor f;
+        place(active ? tid : 0, d, cc);
+        size_t g = tile_src(a, tile, d, cc);
+        if (a.pw_b) {
+            ld_elem_cg(b, a.pw_b + 2 * g);
+            ld_elem_cg(c, a.pw_c + 2 * g);
+        }
+        if (a.pre) ldg_factor(f, a.pre + 4 * size_t(d));
+#pragma unroll 1
+        for (uint32_t e = tid; active && e < CN; e += nthreads) {
+            const uint32_t u = smem_unit(cc, d, K, lc);
+            uint32_t x[8], q[8];
+            lds_elem(x, buf, u);
+            if (e + nthreads < CN) place(e + nthreads, d, cc);
+            g = tile_src(a, tile, d, cc);
             if (a.pw_b) {
-                const size_t g = tile_src(a, tile, d, cc);
-                uint32_t v[8], u[8];
-                ld_elem_cg(v, a.pw_b + 2 * g);
-                ld_elem_cg(u, a.pw_c + 2 * g);
-                mul<F>(x, x, v);
-                sub<F>(x, x, u);
+                mul<F>(x, b, x);
+                ld_elem_cg(b, a.pw_b + 2 * g);
+                sub<F>(x, x, c);
+                ld_elem_cg(c, a.pw_c + 2 * g);
             }
             if (a.pre) {
-                Factor f;
-                ldg_factor(f, a.pre + 4 * size_t(d));
-                mul_factor<F>(x, x, f);
+                mul_high(q, x, f.wq);
+                ZK_LD8("", f.wq, a.pre + 4 * size_t(d) + 2);
+                mul_low_fold<F>(x, x, f.w, q);
+                ZK_LD8("", f.w, a.pre + 4 * size_t(d));
             }
-            sts_elem(buf, s, x);
+            sts_elem(buf, u, x);
         }
         __syncthreads();
     }
@@ -534,14 +606,6 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
     if (STEPS == RADIX2 || (STEPS == EITHER && nthreads > (CN >> 2))) {
         run_stages<F, EARLY>(a, tab, buf, tile, nthreads);
         return;
-    }
-
-    // the thread's entries of the big table are wanted in the last step: into L2
-    // (by single prefetches: the bulk form takes one lane at a time)
-    if (K >= 2 && !a.last && !a.otf && active && tid < (CN >> 2)) {
-        const OutRows o = out_rows<4>(a, tile, (tid >> lc) << 2, tid & (C - 1));
-#pragma unroll
-        for (int i = 0; i < 4; i++) prefetch_l2(o.f + i * o.fstep);
     }
 
     // ---- stages 0 .. K-3
@@ -555,7 +619,7 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
         // the thread's group, and its column's part of the units
         const uint32_t g0 = tid & ((N >> 2) - 1), c0 = col_unit(tid >> (K - 2), K, lc);
         uint32_t shift = K & 1u;  // the step's first stage: entries j 2^shift and (j + q) 2^shift
-#pragma unroll 1
+#pragma unroll
         for (; q > 1; q >>= 2, shift += 2) {
             // rows i0 + {0, q, 2q, 3q}: the stage of distance 2q, then of distance q
             const uint32_t x1 = row_unit(q), x2 = row_unit(2 * q), xt = tab_unit(q << shift);
@@ -564,26 +628,24 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
                 const uint32_t j = b & (q - 1);
                 const uint32_t u0 = c ^ row_unit(4 * b - 3 * j);
                 const uint32_t ta = tab_unit(j << shift), tb = tab_unit(j << (shift + 1));
-                uint32_t v0[8], v1[8], v2[8], v3[8], t[8];
-                Factor w;
+                uint32_t v0[8], v1[8], v2[8], v3[8], t[8], u[8];
+                Factor w, z;
                 lds_elem(v0, buf, u0);
                 lds_elem(v2, buf, u0 ^ x2);
                 lds_factor(w, tab, ta);
-                sum_diff<F>(v0, t, v2);
-                mul_factor<F>(v2, t, w);
                 lds_elem(v1, buf, u0 ^ x1);
                 lds_elem(v3, buf, u0 ^ x1 ^ x2);
-                lds_factor(w, tab, ta ^ xt);
-                sum_diff<F>(v1, t, v3);
-                mul_factor<F>(v3, t, w);
+                lds_factor(z, tab, ta ^ xt);
+                sum_diff<F>(v0, t, v2);
+                sum_diff<F>(v1, u, v3);
+                mul_factor2<F>(v2, t, w, v3, u, z);
                 lds_factor(w, tab, tb);
                 sum_diff<F>(v0, t, v1);
+                sum_diff<F>(v2, u, v3);
                 sts_elem(buf, u0, v0);
-                mul_factor<F>(v1, t, w);
-                sts_elem(buf, u0 ^ x1, v1);
-                sum_diff<F>(v2, t, v3);
                 sts_elem(buf, u0 ^ x2, v2);
-                mul_factor<F>(v3, t, w);
+                mul_factor2<F>(v1, t, w, v3, u, w);
+                sts_elem(buf, u0 ^ x1, v1);
                 sts_elem(buf, u0 ^ x1 ^ x2, v3);
                 g += nthreads;
                 b = g & ((N >> 2) - 1);
@@ -637,7 +699,7 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
                 sts_elem(buf, u0 ^ 1u, x1);
                 sts_elem(buf, u0 ^ 2u, x2);
                 sts_elem(buf, u0 ^ 3u, x3);
-                scale_and_store<F, 4>(a, buf, u0, o, tile, d0, cc);
+                scale_and_store<F, 4, STEPS != EITHER>(a, buf, u0, o, tile, d0, cc);
             }
         }
     } else {
@@ -657,7 +719,7 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
             } else {
                 sts_elem(buf, u0, x0);
                 sts_elem(buf, u0 ^ 1u, x1);
-                scale_and_store<F, 2>(a, buf, u0, o, tile, 0, cc);
+                scale_and_store<F, 2, STEPS != EITHER>(a, buf, u0, o, tile, 0, cc);
             }
         }
     }
@@ -665,11 +727,10 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
 
 // threads per block of schedule variant v for a tile of C x 2^K elements: one
 // per four elements (variant 5: two, one butterfly a thread and stage), at most
-// what the variant's kernel is compiled for
-__host__ __device__ constexpr uint32_t pass_max_threads(int v) { return v == 1 || v == 7 ? 128u : 256u; }
+// 256
 __host__ __device__ constexpr uint32_t pass_threads_for(uint32_t K, uint32_t lc, int v) {
     const uint32_t t = K >= 2 ? 1u << (K + lc - (v == 5 ? 1 : 2)) : 1u << lc;
-    return t < pass_max_threads(v) ? t : pass_max_threads(v);
+    return t < 256u ? t : 256u;
 }
 
 // What a pass kernel is compiled for.  ANY: every argument is a runtime value.

@@ -197,15 +197,14 @@ static zkntt_status fill_uniform(zkntt_field field, void *d, size_t n) {
     return ZKNTT_OK;
 }
 
-// Candidate schedules for one digit split: both twiddle modes, the variants of
-// different kernels (1, 2 and 5; the other numbers share theirs or a smaller
-// register budget that was slower at every size), column caps 1, 0, 2 and 3 (the
-// kernels compiled for a digit first).
+// Candidate schedules for one digit split: both twiddle modes, the two variants of
+// different kernels, column caps 1, 0, 2 and 3 (the kernels compiled for a digit
+// first).
 static void split_candidates(int log_n, const std::vector<int> &d, std::vector<zkntt_plan_options> &out) {
     const int p = int(d.size());
     for (int mode : {ZKNTT_TWIDDLE_PRECOMP, ZKNTT_TWIDDLE_OTF})
         for (int cap : {1, 0, 2, 3})
-            for (int ilp : {1, 2, 5}) {
+            for (int ilp : {1, 5}) {
                 if (p == 1 && (mode == ZKNTT_TWIDDLE_OTF || cap != 3)) continue;
                 zkntt_plan_options o;
                 memset(&o, 0, sizeof o);

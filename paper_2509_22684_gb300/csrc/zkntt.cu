@@ -297,8 +297,8 @@ zkntt_status device_info(DeviceInfo **out) {
     if (!d.init) {
         ZK_CHECK(cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev));
         for (int f = 0; f < NUM_FIELDS; f++)
-            for (int ilp = 1; ilp <= NUM_VARIANTS; ilp++)
-                ZK_CHECK(cudaFuncSetAttribute(field_kernels(f).pass[ilp],
+            for (const void *k : {field_kernels(f).any4, field_kernels(f).any2})
+                ZK_CHECK(cudaFuncSetAttribute(k,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               PASS_MAX_SMEM));
         for (int f = 0; f < NUM_FIELDS; f++)
@@ -531,7 +531,7 @@ zkntt_status set_launch(const PassPlan *ps, PassLaunch *r, int field, Kind kind,
         r->kernel = fixed;
         r->threads = 1 << (ps->K + ps->log_cols - (ps->ilp == 5 ? 1 : 2));
     } else {
-        r->kernel = kk.pass[ps->ilp];
+        r->kernel = ps->ilp == 5 ? kk.any2 : kk.any4;
         r->threads = int(pass_threads_for(uint32_t(ps->K), uint32_t(ps->log_cols), ps->ilp));
     }
     // the twiddle table and the tile buffers
@@ -1131,14 +1131,22 @@ zkntt_status g16_plans(int field, int log_n, G16Plans **out) {
     return ZKNTT_OK;
 }
 
-zkntt_status launch_pointwise(int field, const void *a, const void *b, const void *c,
-                              const void *z_dev, void *h, size_t n, cudaStream_t s) {
+// h = (a b - c) z; z: any 256-bit value in Montgomery form
+zkntt_status launch_pointwise(int field, const void *a, const void *b, const void *c, E8 z, void *h,
+                              size_t n, cudaStream_t s) {
     DeviceInfo *dev;
     zkntt_status st = device_info(&dev);
     if (st != ZKNTT_OK) return st;
-    void *args[] = {&a, &b, &c, &z_dev, &h, &n};
-    return from_cuda(cudaLaunchKernel(field_kernels(field).pointwise,
-                                      dim3(grid_for(n, 256, dev->sms)), dim3(256), args, 0, s));
+    const HostField &F = host_field(field);
+    while (geq8(z, F.p)) sub8(z, z, F.p);
+    const HFactor hf = hfactor(F, z);
+    Factor f;
+    memcpy(f.w, hf.w.data(), 32);
+    memcpy(f.wq, hf.wq.data(), 32);
+    void *args[] = {&a, &b, &c, &f, &h, &n};
+    const int grid = int(std::min<size_t>((n + 127) / 128, size_t(dev->sms) * 5));
+    return from_cuda(
+        cudaLaunchKernel(field_kernels(field).pointwise, dim3(grid), dim3(128), args, 0, s));
 }
 
 }  // namespace
@@ -1410,14 +1418,7 @@ zkntt_status zkntt_groth16_h_ex(zkntt_field field, int log_n, const void *d_a, c
             if ((st = zkntt_execute(G->intt, in[k], sv[k], s))) return st;
         for (int k = 0; k < 3; k++)
             if ((st = zkntt_execute(G->cntt, sv[k], sv[k], s))) return st;
-        uint4 *z = nullptr;
-        zkntt_status sa = pool_alloc(reinterpret_cast<void **>(&z), 32, s);
-        if (sa != ZKNTT_OK) return sa;
-        st = from_cuda(cudaMemcpyAsync(z, G->zinv.data(), 32, cudaMemcpyHostToDevice, s));
-        if (st == ZKNTT_OK) st = launch_pointwise(field, S0, S1, S2, z, d_h, size_t(1) << log_n, s);
-        zkntt_status st2 = from_cuda(cudaFreeAsync(z, s));
-        if (st != ZKNTT_OK) return st;
-        if (st2 != ZKNTT_OK) return st2;
+        if ((st = launch_pointwise(field, S0, S1, S2, G->zinv, d_h, size_t(1) << log_n, s))) return st;
         return zkntt_execute(G->cintt, d_h, d_h, s);
     }
     // fused: cosetINTT_{g^-1}(a, b, c) -> S0, S1, S2 and NTT in place on them, three
@@ -1746,14 +1747,9 @@ zkntt_status zkntt_pointwise(zkntt_field field, const void *d_a, const void *d_b
     if (!z_mont) return ZKNTT_EINVAL;
     if (n == 0) return ZKNTT_OK;
     if (bad_ptr(d_a) || bad_ptr(d_b) || bad_ptr(d_c) || bad_ptr(d_h)) return ZKNTT_EINVAL;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    void *z = nullptr;
-    zkntt_status sa = pool_alloc(&z, 32, s);
-    if (sa != ZKNTT_OK) return sa;
-    zkntt_status st = from_cuda(cudaMemcpyAsync(z, z_mont, 32, cudaMemcpyHostToDevice, s));
-    if (st == ZKNTT_OK) st = launch_pointwise(field, d_a, d_b, d_c, z, d_h, n, s);
-    zkntt_status st2 = from_cuda(cudaFreeAsync(z, s));
-    return st != ZKNTT_OK ? st : st2;
+    E8 z;
+    for (int i = 0; i < 8; i++) z[i] = z_mont[i];
+    return launch_pointwise(field, d_a, d_b, d_c, z, d_h, n, static_cast<cudaStream_t>(stream));
 }
 
 zkntt_status zkntt_mulbench(zkntt_field field, int blocks, int threads, int iters, void *d_sink,
