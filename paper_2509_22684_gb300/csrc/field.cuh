@@ -498,13 +498,14 @@ __device__ __forceinline__ void mul(uint32_t r[8], const uint32_t a[8], const ui
 // of them (2r, and where it is below 2^256 4r, stay under 2^256 - 2^251).  If x is
 // a value in Montgomery form, so is the result: w itself is not in it.
 //
-// Work on the heavy FMA datapath: 43 + 28 wide multiply-adds and 8 low ones for
-// q and x w, and 15 and 6 (BLS12-381: r_0 = 1, r_1 = 2^32 - 1 leave two limbs of
-// 2^256 - r that need no multiply), 21 and 7 (BLS12-377) or 28 and 8 (BN254)
-// for q (2^256 - r), against 112 to 120 wide ones of the Montgomery product.
-// Measured in isolation as above: BLS12-381 80.8 -> 99.1 G products/s, BN254
-// 73.7 -> 89.9, BLS12-377 79.3 -> 95.5.  The price is 64 bytes a twiddle.
-
+// Work on the heavy FMA datapath: 43 + 28 wide multiply-adds and 8 narrow ones for q
+// and x w, and 15 and 6 (BLS12-381: r_1 = 2^32 - 1) or 21 and 7 (BLS12-377, BN254)
+// for q (2^256 - r), whose lowest limb is 2^32 - 1 (r_0 = 1) or 2^28 - 1 (BN254) and
+// takes shifts and a subtraction; against 112 to 120 wide ones of the Montgomery
+// product.  About 135 instructions.  Measured in isolation as above: BLS12-381 80.8
+// -> 95.9 G products/s, BN254 73.7 -> 90, BLS12-377 79.3 -> 95.  A wide multiply-add
+// is issued every 4.5 cycles at best (the datapath holds it for 4), and every other
+// instruction costs about 0.75 cycles beside it.  The price is 64 bytes a twiddle.
 //
 // The chains below are written on named registers: e_c and o_c hold the words
 // of columns of even and odd index, a wide multiply-add's two words side by
@@ -568,7 +569,7 @@ __device__ __forceinline__ void mul(uint32_t r[8], const uint32_t a[8], const ui
     ZK_MAD(e6, e7, x5, w1) ZK_MAD(o5, o6, x5, w0) ZK_MADCL(o7, x5, w2)                             \
     ZK_MAD(e6, e7, x6, w0) ZK_MADL(o7, x6, w1)                                                     \
     ZK_MADL(o7, x7, w0)
-// columns 0..7 of q n added, n = n_j 2^(32 j) + ... + n_7 2^224 (j = 2, 1, 0)
+// columns 0..7 of q n added, n = n_j 2^(32 j) + ... + n_7 2^224 (j = 2, 1)
 #define ZK_ROWS_N2                                                                                 \
     ZK_MAD(e2, e3, q0, n2) ZK_MADC(e4, e5, q0, n4) ZK_MADC(e6, e7, q0, n6)                         \
     ZK_MAD(o3, o4, q0, n3) ZK_MADC(o5, o6, q0, n5) ZK_MADCL(o7, q0, n7)                            \
@@ -589,20 +590,6 @@ __device__ __forceinline__ void mul(uint32_t r[8], const uint32_t a[8], const ui
     ZK_MAD(e6, e7, q4, n2) ZK_MAD(o5, o6, q4, n1) ZK_MADCL(o7, q4, n3)                             \
     ZK_MAD(e6, e7, q5, n1) ZK_MADL(o7, q5, n2)                                                     \
     ZK_MADL(o7, q6, n1)
-#define ZK_ROWS_N0                                                                                 \
-    ZK_MAD(e0, e1, q0, n0) ZK_MADC(e2, e3, q0, n2) ZK_MADC(e4, e5, q0, n4)                         \
-    ZK_MADC(e6, e7, q0, n6) ZK_MAD(o1, o2, q0, n1) ZK_MADC(o3, o4, q0, n3)                         \
-    ZK_MADC(o5, o6, q0, n5) ZK_MADCL(o7, q0, n7)                                                   \
-    ZK_MAD(e2, e3, q1, n1) ZK_MADC(e4, e5, q1, n3) ZK_MADC(e6, e7, q1, n5)                         \
-    ZK_MAD(o1, o2, q1, n0) ZK_MADC(o3, o4, q1, n2) ZK_MADC(o5, o6, q1, n4) ZK_MADCL(o7, q1, n6)    \
-    ZK_MAD(e2, e3, q2, n0) ZK_MADC(e4, e5, q2, n2) ZK_MADC(e6, e7, q2, n4)                         \
-    ZK_MAD(o3, o4, q2, n1) ZK_MADC(o5, o6, q2, n3) ZK_MADCL(o7, q2, n5)                            \
-    ZK_MAD(e4, e5, q3, n1) ZK_MADC(e6, e7, q3, n3) ZK_MAD(o3, o4, q3, n0)                          \
-    ZK_MADC(o5, o6, q3, n2) ZK_MADCL(o7, q3, n4)                                                   \
-    ZK_MAD(e4, e5, q4, n0) ZK_MADC(e6, e7, q4, n2) ZK_MAD(o5, o6, q4, n1) ZK_MADCL(o7, q4, n3)     \
-    ZK_MAD(e6, e7, q5, n1) ZK_MAD(o5, o6, q5, n0) ZK_MADCL(o7, q5, n2)                             \
-    ZK_MAD(e6, e7, q6, n0) ZK_MADL(o7, q6, n1)                                                     \
-    ZK_MADL(o7, q7, n0)
 
 // q = floor(x y / 2^256), less at most 1 (bound above)
 __device__ __forceinline__ void mul_high(uint32_t q[8], const uint32_t x[8], const uint32_t y[8]) {
@@ -641,6 +628,16 @@ __device__ __forceinline__ void mul_low_fold(uint32_t t[8], const uint32_t x[8],
     "subc.cc.u32 e2, q1, q2;\n\tsubc.cc.u32 e3, q2, q3;\n\t"                     \
     "subc.cc.u32 e4, q3, q4;\n\tsubc.cc.u32 e5, q4, q5;\n\t"                     \
     "subc.cc.u32 e6, q5, q6;\n\tsubc.u32 e7, q6, q7;\n\t"
+#define ZK_LOW_Q28  /* q (2^28 - 1) = (q << 28) - q */                              \
+    ".reg .u32 s<8>;\n\t"                                                          \
+    "shl.b32 s0, q0, 28;\n\tshf.l.wrap.b32 s1, q0, q1, 28;\n\t"                   \
+    "shf.l.wrap.b32 s2, q1, q2, 28;\n\tshf.l.wrap.b32 s3, q2, q3, 28;\n\t"        \
+    "shf.l.wrap.b32 s4, q3, q4, 28;\n\tshf.l.wrap.b32 s5, q4, q5, 28;\n\t"        \
+    "shf.l.wrap.b32 s6, q5, q6, 28;\n\tshf.l.wrap.b32 s7, q6, q7, 28;\n\t"        \
+    "sub.cc.u32 e0, s0, q0;\n\tsubc.cc.u32 e1, s1, q1;\n\t"                      \
+    "subc.cc.u32 e2, s2, q2;\n\tsubc.cc.u32 e3, s3, q3;\n\t"                     \
+    "subc.cc.u32 e4, s4, q4;\n\tsubc.cc.u32 e5, s5, q5;\n\t"                     \
+    "subc.cc.u32 e6, s6, q6;\n\tsubc.u32 e7, s7, q7;\n\t"
 #define ZK_LOW_TAIL                                                                \
     "mov.u32 %0, e0;\n\t"                                                          \
     "add.cc.u32 %1, e1, o1;\n\taddc.cc.u32 %2, e2, o2;\n\t"                      \
@@ -659,11 +656,12 @@ __device__ __forceinline__ void mul_low_fold(uint32_t t[8], const uint32_t x[8],
         asm(ZK_LOW_HEAD ZK_LOW_Q ZK_ROW_LOW_ADD ZK_ROWS_LOW ZK_ROWS_N1 ZK_LOW_TAIL
             ZK_LOW_OPERANDS(0, ~F::P1));
     } else {
-        asm(ZK_LOW_HEAD ZK_ROW_LOW_NEW ZK_ROWS_LOW ZK_ROWS_N0 ZK_LOW_TAIL
-            ZK_LOW_OPERANDS(0u - F::P0, ~F::P1));
+        asm(ZK_LOW_HEAD ZK_LOW_Q28 ZK_ROW_LOW_ADD ZK_ROWS_LOW ZK_ROWS_N1 ZK_LOW_TAIL
+            ZK_LOW_OPERANDS(0, ~F::P1));
     }
 #undef ZK_LOW_HEAD
 #undef ZK_LOW_Q
+#undef ZK_LOW_Q28
 #undef ZK_LOW_TAIL
 #undef ZK_LOW_OPERANDS
 }

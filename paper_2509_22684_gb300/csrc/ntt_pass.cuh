@@ -536,9 +536,9 @@ __device__ __forceinline__ void run_stages(const PassArgs &a, const uint4 *tab, 
 // synchronised since), with `nthreads` threads of the block (threads at or
 // beyond nthreads only take part in the barriers).  The block does not
 // synchronise at the end: `buf` may be written again after a barrier.
-// EARLY: in the radix-2 form, whether the output factors are read before the stages
-// (a thread has one pair of each stage).
-template <class F, Steps STEPS, bool EARLY = false>
+// COMPILED: the sizes are constants and all threads of the block have one group
+// (radix 4) or pair (radix 2) in each step.
+template <class F, Steps STEPS, bool COMPILED = false>
 __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, uint4 *buf,
                                          uint32_t tile, uint32_t nthreads) {
     const uint32_t K = a.K, lc = a.log_cols;
@@ -604,20 +604,64 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
     }
 
     if (STEPS == RADIX2 || (STEPS == EITHER && nthreads > (CN >> 2))) {
-        run_stages<F, EARLY>(a, tab, buf, tile, nthreads);
+        run_stages<F, COMPILED>(a, tab, buf, tile, nthreads);
         return;
+    }
+
+    // With 10 bits and more two blocks fit an SM, too few to wait for the entries of
+    // the big table that the last step wants: into L2 (2^20, digits 10 and 10: 157 ->
+    // 148 us; no gain for smaller digits).
+    if (K >= 10 && !a.last && !a.otf && active && tid < (CN >> 2)) {
+        const OutRows o = out_rows<4>(a, tile, (tid >> lc) << 2, tid & (C - 1));
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(o.f + i * o.fstep));
     }
 
     // ---- stages 0 .. K-3
     if (K > 2) {
         uint32_t q = N >> 2;  // distance of a radix-4 step's rows
-        if (K & 1u) {
-            radix2_stage<F>(buf, tab, N >> 1, K, lc, tid, nthreads);
-            __syncthreads();
-            q >>= 1;
-        }
         // the thread's group, and its column's part of the units
         const uint32_t g0 = tid & ((N >> 2) - 1), c0 = col_unit(tid >> (K - 2), K, lc);
+        // After a step at distance q that the step at q/4 or q/8 follows: at q <= 32 a
+        // warp's groups, 32 consecutive ones, are made of rows of its own, at this
+        // step and the next; a column's threads exchange rows otherwise.  The last
+        // step (columns fastest) reads every column.
+        auto sync = [&](uint32_t q, bool to_last) {
+            if (to_last && (lc > 0 || q > 32)) __syncthreads();
+            else if (q <= 32) __syncwarp();
+            else if (COMPILED && lc > 0)
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + (tid >> (K - 2))), "r"(N >> 2) : "memory");
+            else __syncthreads();
+        };
+        if (K & 1u) {
+            // the first stage alone, on the rows of a step at distance N/4
+            const uint32_t x1 = row_unit(q), x2 = row_unit(2 * q), xt = tab_unit(q);
+            uint32_t g = tid, b = g0, c = c0;
+            while (active && g < (CN >> 2)) {
+                const uint32_t u0 = c ^ row_unit(b), ta = tab_unit(b);
+                uint32_t v0[8], v1[8], v2[8], v3[8], t[8], u[8];
+                Factor w, z;
+                lds_elem(v0, buf, u0);
+                lds_elem(v2, buf, u0 ^ x2);
+                lds_factor(w, tab, ta);
+                lds_elem(v1, buf, u0 ^ x1);
+                lds_elem(v3, buf, u0 ^ x1 ^ x2);
+                lds_factor(z, tab, ta ^ xt);
+                sum_diff<F>(v0, t, v2);
+                sts_elem(buf, u0, v0);
+                sum_diff<F>(v1, u, v3);
+                sts_elem(buf, u0 ^ x1, v1);
+                mul_factor2<F>(v2, t, w, v3, u, z);
+                sts_elem(buf, u0 ^ x2, v2);
+                sts_elem(buf, u0 ^ x1 ^ x2, v3);
+                g += nthreads;
+                b = g & ((N >> 2) - 1);
+                c = col_unit(g >> (K - 2), K, lc);
+            }
+            sync(q, K == 3);
+            q >>= 1;
+        }
         uint32_t shift = K & 1u;  // the step's first stage: entries j 2^shift and (j + q) 2^shift
 #pragma unroll
         for (; q > 1; q >>= 2, shift += 2) {
@@ -651,11 +695,7 @@ __device__ __forceinline__ void run_tile(const PassArgs &a, const uint4 *tab, ui
                 b = g & ((N >> 2) - 1);
                 c = col_unit(g >> (K - 2), K, lc);
             }
-            // at q <= 32 a warp's groups, 32 consecutive ones, are made of rows
-            // of its own, at this step and the next: only the last step (columns
-            // fastest) reads another warp's
-            if (q > 32 || q == 4) __syncthreads();
-            else __syncwarp();
+            sync(q, q == 4);
         }
     }
 
