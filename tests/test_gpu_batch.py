@@ -258,12 +258,12 @@ def test_groth16_contract_signature_runs_the_fused_form():
     assert np.array_equal(to_host(h), ref.groth16_h_mont(F, A, B, C))
 
 
-@pytest.mark.parametrize("L", [16, 17, 19])
+@pytest.mark.parametrize("L", [1, 5, 16, 17, 19])
 @pytest.mark.parametrize("F", [fld.BLS12_381, fld.BN254, fld.BLS12_377], ids=lambda f: f.name)
-def test_groth16_forms_agree_across_the_size_rule(F, L):
-    """The fused sequence is one persistent launch below 2^17 and passes of the
-    compiled kernels from there on: both, called and replayed from a graph, equal
-    the seven transforms and the pointwise step issued one by one."""
+def test_groth16_forms_agree(F, L):
+    """The fused sequence, three transforms a launch and its launches chained,
+    called and replayed from a graph, equals the seven transforms and the
+    pointwise step issued one by one."""
     import torch
     import paper_2509_22684_gb300 as zk
     a, b, c = (rand_dev(F, L, 900 + 10 * L + k)[1] for k in range(3))

@@ -115,6 +115,23 @@ def test_pointwise(F):
     assert got == want
 
 
+@pytest.mark.parametrize("F", FIELDS, ids=lambda f: f.name)
+@pytest.mark.parametrize("n", [1, 127, 129, 100003])
+def test_pointwise_sizes_and_in_place(F, n):
+    """One element, a block's edges, a grid that loops, the output over an input,
+    and the extreme values of the constant."""
+    import paper_2509_22684_gb300 as zk
+    A, B, C = (limbs_to_ints(uniform_elements(F.r, n, s)) for s in (24, 25, 26))
+    r = F.r
+    for k, v in enumerate(_edge_values(F)[:n]):
+        A[k], C[k] = v, r - 1 - v
+    for z in (0, 1, r - 1):
+        a, b, c = (to_dev(ints_to_limbs(v)) for v in (A, B, C))
+        zk.pointwise(F.name, a, b, c, z, out=a)
+        want = [F.mont_mul((F.mont_mul(x, y) - w) % r, z) for x, y, w in zip(A, B, C)]
+        assert limbs_to_ints(to_host(a)) == want
+
+
 def test_field_info_matches_oracle():
     import paper_2509_22684_gb300 as zk
     for F in FIELDS:

@@ -237,6 +237,38 @@ def test_kernel_variants(F, kind, variant, digits, cols):
     assert np.array_equal(got, want), first_mismatch(got, want)
 
 
+def _edge_dev(F, L):
+    """Elements 0, 1, r - 1, r - 2, R and their neighbours in a random order: sums
+    and differences at both ends of the residues' range."""
+    from workloads import ints_to_limbs, splitmix64
+    r = F.r
+    edge = ints_to_limbs([0, 1, 2, r - 1, r - 2, F.R % r, r >> 1, (r >> 1) + 1])
+    X = np.ascontiguousarray(edge[(splitmix64(55, 0, 1 << L) % 8).astype(np.int64)])
+    return X, to_dev(X)
+
+
+@pytest.mark.parametrize("F", FIELDS, ids=lambda f: f.name)
+@pytest.mark.parametrize("variant", [1, 5])
+@pytest.mark.parametrize("digits", [(5, 5), (6, 7), (7, 6), (8, 8), (9, 8), (8, 9), (10, 9), (9, 10),
+                                    (5, 10, 5), (8, 4, 8)])
+def test_compiled_kernels_equal_the_general_one(F, variant, digits):
+    """Digits of 5 to 10 bits in tiles of two columns (10 bits: one) run in kernels
+    compiled for them, in tiles of another width in the general one: every kind,
+    with tables and on the fly, from two vectors, against the oracle."""
+    L = sum(digits)
+    compiled = [1 if k == 10 else 2 for k in digits]
+    general = [2 if k == 10 else 4 if k < 9 else 1 for k in digits]
+    inputs = [rand_dev(F, L, 3000 + L), _edge_dev(F, L)]
+    for kind in KINDS:
+        want = [_oracle(F, X, kind) for X, _ in inputs]
+        for mode in ("precomp", "otf"):
+            for cols in (compiled, general):
+                with _plan(F, L, kind, twiddle_mode=mode, digits=digits, cols=cols, ilp=variant) as p:
+                    for (_, x), w in zip(inputs, want):
+                        got = to_host(p.execute(x))
+                        assert np.array_equal(got, w), (kind, mode, cols, first_mismatch(got, w))
+
+
 def test_tuner_picks_a_schedule_that_stays_exact(tmp_path, monkeypatch):
     import paper_2509_22684_gb300 as zk
     monkeypatch.setenv("ZKNTT_TUNE_CACHE", str(tmp_path / "tune.jsonl"))
