@@ -453,7 +453,7 @@ def serve_bench(zk, torch, field: str, n_requests: int, loads, solo_log_n=None) 
 
 
 def groth16_only(args) -> None:
-    """Groth16 H at 2^L: the fused persistent launch in a CUDA graph and the
+    """Groth16 H at 2^L: the fused launches in a CUDA graph and the
     seven transforms + pointwise issued separately, both after warm-up, with
     CUDA events (one JSON line; rank 0 only)."""
     import numpy as np
@@ -808,7 +808,8 @@ def main():
     ap.add_argument("--sweep-sizes", default="16,20,22,24,26")
     ap.add_argument("--sweep-fields", default="bls12_381_fr,bn254_fr,bls12_377_fr")
     ap.add_argument("--variant", type=int, default=0,
-                    help="force pass-kernel variant V on the shipped digit split (study runs)")
+                    help="force pass-kernel variant V on the shipped digit split (study runs): "
+                         "1 two stages at a time, 5 one butterfly a thread")
     ap.add_argument("--calibrate", action="store_true",
                     help="print the multiply-form and product rates instead")
     ap.add_argument("--sharded", type=int, default=0, metavar="G",

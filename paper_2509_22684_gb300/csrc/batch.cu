@@ -20,9 +20,12 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
 // segment; status: sticky per-device error word read by the host.  Thread 0
 // claims the block's next work item while the current tile is processed, so
 // the atomic's round trip is hidden behind the tile; the claimed index waits in
-// shared memory, which keeps the tile routine's register budget (64, for four
-// blocks of 256 per SM) free of bookkeeping.  One kernel per field: the tile
-// routine is inlined and its constants are immediates.
+// shared memory, which keeps the tile routine's registers free of bookkeeping.  One
+// kernel per field: the tile routine is inlined and its constants are immediates.
+// Bound by the products as the pass kernel is, and by its runtime sizes (a digit
+// compiled in took 1865 us instead of 1872, for five times the code).  64 uneven
+// transforms of 2^10..2^20, two fields: 2669 us with the Montgomery product and
+// radix-2 steps, now 1824.
 template <class F>
 __global__ void __launch_bounds__(BATCH_THREADS, BATCH_MIN_BLOCKS)
     batch_kernel(const __grid_constant__ BatchTable tab, uint32_t *ctrl, uint32_t *done,

@@ -25,8 +25,16 @@
 // take the stages one by one, one butterfly a thread.
 // The difference x - y is formed as x + r - y with no conditional correction:
 // it only feeds the product, which takes any x below 2r.
-// All sizes (K, C, the stride) are runtime values: one kernel per field serves
-// every digit size.
+// Digits of 5 to 10 bits in the usual tile width have kernels compiled for them;
+// every other digit and width is served by kernels whose sizes are runtime values.
+//
+// What bounds it: the heavy FMA datapath and the issue of everything beside it.  A
+// pass of 8 bits makes 3.25 products an element in its stages and one for the output
+// factor, 133 instructions each, 86 of them wide multiply-adds that hold the datapath
+// for four cycles.  At 2^24 (three passes of 8 bits, 2590 us on GB300; 4537 with
+// Montgomery products and radix-2 steps) the datapath is busy 67 to 72% of the
+// cycles.  Memory costs little: with neither vectors nor inter-pass factors read, the
+// first pass takes 926 us instead of 985.
 //
 // Values are residues in [0, 2r) throughout; the last pass brings its outputs
 // below r.
@@ -251,9 +259,7 @@ __device__ __forceinline__ void scale_and_store(const PassArgs &a, const uint4 *
                                                 uint32_t cc) {
     if (o.f) {
         Factor v;
-        // (an entry of the big table is read once: it takes no place in L1)
-        if (a.last) ldg_factor(v, o.f);
-        else ldg_factor_stream(v, o.f);
+        ldg_out_factor(v, a, o.f);
         const uint4 *f = o.f;
 #pragma unroll 1
         for (uint32_t i = 0; i < R; i++) {
@@ -776,8 +782,8 @@ __host__ __device__ constexpr uint32_t pass_threads_for(uint32_t K, uint32_t lc,
 // What a pass kernel is compiled for.  ANY: every argument is a runtime value.
 // The others: a digit of K bits in tiles of fixed_cols(K) columns; a strided pass
 // with precomputed twiddles, its input without factors (STRIDED) or with
-// (STRIDED_PRE: input scales or the pointwise step), or with twiddles on the fly (STRIDED_OTF); the last pass without
-// output factors (LAST) or with (LAST_POST).  With these fixed the index
+// (STRIDED_PRE: input scales or the pointwise step), or with twiddles on the fly
+// (STRIDED_OTF); the last pass without output factors (LAST) or with (LAST_POST).  With these fixed the index
 // arithmetic of a tile shrinks: 803 -> 692 instructions an element in the last
 // pass of 2^22, which was 691 us and is 642 (BLS12-381, digits 8, 7, 7).  (With
 // the digit alone fixed and the factors left to the arguments 2^22 took 648, 2^12
@@ -786,7 +792,8 @@ enum Kind { ANY, STRIDED, STRIDED_PRE, STRIDED_OTF, LAST, LAST_POST, NUM_KINDS }
 
 // log2 of the columns of the tiles of the compiled digits: two, so that global
 // memory is read and written in 64-byte pieces; one where two make a tile and
-// table of which only one would fit an SM
+// table of which only one would fit an SM.  (Four or eight columns for digits of 6
+// and 7 bits: 2^24 2591 -> 2705 us, 2^26 11417 -> 11641.)
 __host__ __device__ constexpr int fixed_cols(int K) { return K < 10 ? 1 : 0; }
 
 template <int K, Kind KIND>
