@@ -9,7 +9,7 @@
 //    and the columns per block;
 //  * resident twiddle tables per plan, generated on the device;
 //  * stream-ordered execution, the persistent batch launch and the Groth16 H
-//    sequence (Fig. 2 of the paper).
+//    sequence (Fig. 2 of the paper), three transforms a launch.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -94,35 +94,37 @@ uint32_t sub8(E8 &r, const E8 &a, const E8 &b) {
     return c ? 1u : 0u;
 }
 
-// SOS: full 512-bit product, then eight word-wise reductions
+// Montgomery product on four 64-bit words, a word of b and its reduction at a time
+// (the tables of a plan take some 10^4 of them)
+using u128 = unsigned __int128;
 E8 hmul(const HostField &F, const E8 &a, const E8 &b) {
-    uint32_t t[17] = {0};
-    for (int i = 0; i < 8; i++) {
-        uint64_t carry = 0;
-        for (int j = 0; j < 8; j++) {
-            uint64_t v = uint64_t(a[i]) * b[j] + t[i + j] + carry;
-            t[i + j] = uint32_t(v);
-            carry = v >> 32;
+    uint64_t x[4], y[4], p[4], np, t[5] = {0};
+    memcpy(x, a.data(), 32);
+    memcpy(y, b.data(), 32);
+    memcpy(p, F.p.data(), 32);
+    memcpy(&np, F.ninv.data(), 8);
+    for (int i = 0; i < 4; i++) {
+        u128 v = 0;
+        for (int j = 0; j < 4; j++) {
+            v += u128(x[j]) * y[i] + t[j];
+            t[j] = uint64_t(v);
+            v >>= 64;
         }
-        t[i + 8] = uint32_t(carry);
-    }
-    for (int i = 0; i < 8; i++) {
-        uint32_t m = t[i] * F.rp;
-        uint64_t carry = 0;
-        for (int j = 0; j < 8; j++) {
-            uint64_t v = uint64_t(m) * F.p[j] + t[i + j] + carry;
-            t[i + j] = uint32_t(v);
-            carry = v >> 32;
+        v += t[4];
+        t[4] = uint64_t(v);
+        const uint64_t top = uint64_t(v >> 64), m = t[0] * np;
+        v = u128(m) * p[0] + t[0];
+        for (int j = 1; j < 4; j++) {
+            v = (v >> 64) + u128(m) * p[j] + t[j];
+            t[j - 1] = uint64_t(v);
         }
-        for (int k = i + 8; carry && k < 17; k++) {
-            uint64_t v = uint64_t(t[k]) + carry;
-            t[k] = uint32_t(v);
-            carry = v >> 32;
-        }
+        v = (v >> 64) + t[4];
+        t[3] = uint64_t(v);
+        t[4] = top + uint64_t(v >> 64);
     }
     E8 r;
-    for (int i = 0; i < 8; i++) r[i] = t[8 + i];
-    if (t[16] || geq8(r, F.p)) sub8(r, r, F.p);
+    memcpy(r.data(), t, 32);
+    if (t[4] || geq8(r, F.p)) sub8(r, r, F.p);
     return r;
 }
 
@@ -142,15 +144,30 @@ E8 hmul_low(const E8 &a, const E8 &b) {
 
 // A factor table entry of w, given in Montgomery form as m = w R mod p: the
 // integer w and floor(w R / p).  w R = floor(w R / p) p + m, so modulo R the
-// quotient is -m p^-1, and it is below R.
+// quotient is -m p^-1, and it is below R: the multipliers of the reduction of m
+// are its words, and what the reduction leaves is w.
 struct HFactor {
     E8 w, wq;
 };
 
 HFactor hfactor(const HostField &F, const E8 &m) {
-    E8 one{};
-    one[0] = 1;
-    return {hmul(F, m, one), hmul_low(m, F.ninv)};
+    uint64_t t[4], p[4], np, q[4];
+    memcpy(t, m.data(), 32);
+    memcpy(p, F.p.data(), 32);
+    memcpy(&np, F.ninv.data(), 8);
+    for (int i = 0; i < 4; i++) {
+        q[i] = t[0] * np;
+        u128 v = u128(q[i]) * p[0] + t[0];
+        for (int j = 1; j < 4; j++) {
+            v = (v >> 64) + u128(q[i]) * p[j] + t[j];
+            t[j - 1] = uint64_t(v);
+        }
+        t[3] = uint64_t(v >> 64);  // (the sum stays below p)
+    }
+    HFactor f;
+    memcpy(f.w.data(), t, 32);
+    memcpy(f.wq.data(), q, 32);
+    return f;
 }
 
 E8 hsub(const HostField &F, const E8 &a, const E8 &b) {
@@ -950,7 +967,7 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
     // The batch kernel runs 256 threads a block whatever the tile, so a tile of
     // C x 2^K elements with C x 2^K / 4 < 256 leaves threads idle.  Each pass
     // therefore takes the widest tile up to 2^BATCH_TILE_BITS elements (32 KiB,
-    // so four blocks fit an SM's shared memory; an 11-bit digit keeps its
+    // so three blocks fit an SM's shared memory; an 11-bit digit keeps its
     // 2^11-element tile), narrowed toward the plan's own width only while the
     // pass has fewer tiles than one wave of resident blocks (the plan's tables
     // do not depend on the tile width).
