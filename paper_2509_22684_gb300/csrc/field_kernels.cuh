@@ -16,11 +16,12 @@ const void *fixed_kernel() {
     return (const void *)&ntt_pass_kernel<F, T, B, RADIX4, K, KIND>;
 }
 
-// the same one butterfly a thread and stage, for small transforms: 128 registers
+// the same one butterfly a thread and stage, in tiles of one column, for small
+// transforms: 128 registers
 template <class F, int K, Kind KIND>
 const void *wide_kernel() {
-    constexpr int T = 1 << (K + fixed_cols(K) - 1);
-    return (const void *)&ntt_pass_kernel<F, T, 512 / T, RADIX2, K, KIND>;
+    constexpr int T = 1 << (K + fixed_cols(K, RADIX2) - 1);
+    return (const void *)&ntt_pass_kernel<F, T, T >= 32 ? 512 / T : 16, RADIX2, K, KIND>;
 }
 
 template <class F, int K>
@@ -49,6 +50,7 @@ FieldKernels make_field_kernels() {
     set_wide<F, 6>(k);
     set_wide<F, 7>(k);
     set_wide<F, 8>(k);
+    set_wide<F, 9>(k);
     set_fixed<F, 5>(k);
     set_fixed<F, 6>(k);
     set_fixed<F, 7>(k);

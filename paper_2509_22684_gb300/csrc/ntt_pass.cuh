@@ -488,9 +488,10 @@ __device__ __forceinline__ void radix2_stage(uint4 *buf, const uint4 *tab, uint3
 // output: for transforms with few warps in flight, whose time is the chain of
 // products of one thread.  A digit of K bits is a chain of K - 1 products and two
 // independent ones for the output factors, where the radix-4 steps make up to
-// 2 K + 1 (2^12, digits 6 and 6: 12.4 -> 9.9 us, 2^14 14.4 -> 12.2, 2^15 16.4 ->
-// 14.4; 2^16, with a warp for every scheduler of the GPU, 17.2 -> 20.5).  EARLY: read the output
-// factors before the stages (32 registers held across them).
+// 2 K + 1 (2^12, digits 6 and 6: 14.3 -> 10.5 us, 2^14 16.4 -> 13.6, 2^15, 7 and 8,
+// 16.5 -> 12.8, 2^16, 7 and 9, 18.4 -> 16.7; 2^17, with two warps for every scheduler
+// of the GPU, 24.9 -> 31.0).  EARLY: read the output factors before the stages (32
+// registers held across them).
 template <class F, bool EARLY>
 __device__ __forceinline__ void run_stages(const PassArgs &a, const uint4 *tab, uint4 *buf,
                                            uint32_t tile, uint32_t nthreads) {
@@ -507,8 +508,9 @@ __device__ __forceinline__ void run_stages(const PassArgs &a, const uint4 *tab, 
     for (uint32_t h = 1u << (K - 1); h >= 2; h >>= 1) {
         radix2_stage<F>(buf, tab, h, K, lc, tid, nthreads);
         // at h <= 32 a warp's pairs, 32 consecutive ones, are made of rows of its
-        // own, at this stage and the next; the last (columns fastest) reads others'
-        if (h > 32 || h == 2) __syncthreads();
+        // own, at this stage and the next; the last (columns fastest) reads others',
+        // but of one column
+        if (h > 32 || (h == 2 && lc > 0)) __syncthreads();
         else __syncwarp();
     }
 #pragma unroll 1
@@ -780,7 +782,7 @@ __host__ __device__ constexpr uint32_t pass_threads_for(uint32_t K, uint32_t lc,
 }
 
 // What a pass kernel is compiled for.  ANY: every argument is a runtime value.
-// The others: a digit of K bits in tiles of fixed_cols(K) columns; a strided pass
+// The others: a digit of K bits in tiles of fixed_cols columns; a strided pass
 // with precomputed twiddles, its input without factors (STRIDED) or with
 // (STRIDED_PRE: input scales or the pointwise step), or with twiddles on the fly
 // (STRIDED_OTF); the last pass without output factors (LAST) or with (LAST_POST).  With these fixed the index
@@ -792,15 +794,18 @@ enum Kind { ANY, STRIDED, STRIDED_PRE, STRIDED_OTF, LAST, LAST_POST, NUM_KINDS }
 
 // log2 of the columns of the tiles of the compiled digits: two, so that global
 // memory is read and written in 64-byte pieces; one where two make a tile and
-// table of which only one would fit an SM.  (Four or eight columns for digits of 6
+// table of which only one would fit an SM, and for one butterfly a thread, where
+// twice the blocks matter more (2^12 12.6 -> 10.5 us, 2^15 16.4 -> 12.8).  (Four or eight columns for digits of 6
 // and 7 bits: 2^24 2591 -> 2705 us, 2^26 11417 -> 11641.)
-__host__ __device__ constexpr int fixed_cols(int K) { return K < 10 ? 1 : 0; }
+__host__ __device__ constexpr int fixed_cols(int K, Steps steps = RADIX4) {
+    return K < 10 && steps == RADIX4 ? 1 : 0;
+}
 
-template <int K, Kind KIND>
+template <int K, Kind KIND, Steps STEPS>
 __device__ __forceinline__ void fix_args(PassArgs &a) {
     if (KIND == ANY) return;
     a.K = K;
-    a.log_cols = fixed_cols(K);
+    a.log_cols = fixed_cols(K, STEPS);
     a.last = KIND == LAST || KIND == LAST_POST;
     a.otf = KIND == STRIDED_OTF;
     if (KIND != STRIDED_PRE) a.pre = a.pw_b = a.pw_c = nullptr;
@@ -815,7 +820,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
     ntt_pass_kernel(const PassArgs args, const __grid_constant__ PassVectors vec) {
     extern __shared__ uint4 smem[];
     PassArgs a = args;
-    fix_args<K, KIND>(a);
+    fix_args<K, KIND, STEPS>(a);
     const uint32_t nthreads = KIND == ANY ? blockDim.x : THREADS;
     const uint32_t units = tile_units(1u << (a.K + a.log_cols));
     uint4 *tab = smem, *buf = smem + 4 * tab_entries(a.K);

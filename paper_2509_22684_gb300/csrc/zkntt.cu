@@ -487,8 +487,11 @@ void default_digits(int L, int *passes, int k[4]) {
     }
 }
 
-// interleaved butterflies per thread in the stage loop (planner default)
-constexpr int DEFAULT_ILP = 1;
+// The variant without a tuned schedule: two stages at a time, but one butterfly a
+// thread (5) for a transform of one pass up to 2^9, which is one block and waits on
+// its own products (2^3 8.2 -> 6.2 us, 2^6 10.3 -> 6.2, 2^9 12.3 -> 10.3; one block
+// of 2^10 16.4 -> 18.5).
+int default_ilp(int L, int passes) { return passes == 1 && L <= 9 ? 5 : 1; }
 
 int default_log_cols(int K, int span_bits) {
     // tile of C x 2^K elements, at most 2^11 elements (64 KiB); C <= 8 and
@@ -544,7 +547,7 @@ zkntt_status split_tables(zkntt_plan_s *P, const HostField &F, const E8 &base, i
 zkntt_status set_launch(const PassPlan *ps, PassLaunch *r, int field, Kind kind, int sms) {
     const FieldKernels &kk = field_kernels(field);
     const void *fixed = (ps->ilp == 5 ? kk.wide : kk.fixed)[ps->K][kind];
-    if (ps->log_cols == fixed_cols(ps->K) && fixed) {
+    if (ps->log_cols == fixed_cols(ps->K, ps->ilp == 5 ? RADIX2 : RADIX4) && fixed) {
         r->kernel = fixed;
         r->threads = 1 << (ps->K + ps->log_cols - (ps->ilp == 5 ? 1 : 2));
     } else {
@@ -578,7 +581,7 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
     // ---- schedule
     int k[4] = {0, 0, 0, 0}, cols[4] = {-1, -1, -1, -1};
     int mode = ZKNTT_TWIDDLE_AUTO;
-    int ilp = DEFAULT_ILP;
+    int ilp = 0;
     default_digits(L, &P->passes, k);
     // tuned schedules (shipped with the library or from ZKNTT_TUNE_CACHE) are
     // used unless the caller opts out (use_tuner < 0) or forces a split
@@ -615,6 +618,7 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         ilp = opts->ilp;
     }
     const int p = P->passes;
+    if (!ilp) ilp = default_ilp(L, p);
     if (mode == ZKNTT_TWIDDLE_AUTO && p > 1) {
         // Precomputed inter-pass tables (pass i: 2^(K_i + lo_bits_i) entries of
         // 64 bytes; pass 1's is n entries) unless they would not fit beside the input,
@@ -968,16 +972,17 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
     // C x 2^K elements with C x 2^K / 4 < 256 leaves threads idle.  Each pass
     // therefore takes the widest tile up to 2^BATCH_TILE_BITS elements (32 KiB,
     // so three blocks fit an SM's shared memory; an 11-bit digit keeps its
-    // 2^11-element tile), narrowed toward the plan's own width only while the
-    // pass has fewer tiles than one wave of resident blocks (the plan's tables
-    // do not depend on the tile width).
+    // 2^11-element tile), narrowed toward the plan's own width, not below two
+    // columns (64 transforms of 2^10..2^16, whose plans have tiles of one: 250 us,
+    // narrowed to one 328), only while the pass has fewer tiles than one wave of
+    // resident blocks (the plan's tables do not depend on the tile width).
     const uint64_t wave = uint64_t(dev->sms) * BATCH_WAVE_BLOCKS;
     auto batch_log_cols = [&](const zkntt_plan_s *P, int i) {
         const PassPlan &ps = P->ps[i];
         const int span = (i == P->passes - 1) ? ps.hi_bits : ps.lo_bits;
         const int cap = std::max(BATCH_TILE_BITS, ps.K);
         int lc = std::max(0, std::min({3, cap - ps.K, span}));
-        while (lc > ps.log_cols && (uint64_t(1) << (P->log_n - ps.K - lc)) < wave) lc--;
+        while (lc > std::max(ps.log_cols, 1) && (uint64_t(1) << (P->log_n - ps.K - lc)) < wave) lc--;
         return lc;
     };
     auto batch_tiles = [&](const zkntt_plan_s *P, int i) {

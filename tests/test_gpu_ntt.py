@@ -250,14 +250,15 @@ def _edge_dev(F, L):
 @pytest.mark.parametrize("F", FIELDS, ids=lambda f: f.name)
 @pytest.mark.parametrize("variant", [1, 5])
 @pytest.mark.parametrize("digits", [(5, 5), (6, 7), (7, 6), (8, 8), (9, 8), (8, 9), (10, 9), (9, 10),
-                                    (5, 10, 5), (8, 4, 8)])
+                                    (5, 10, 5), (8, 4, 8), (7, 9)])
 def test_compiled_kernels_equal_the_general_one(F, variant, digits):
-    """Digits of 5 to 10 bits in tiles of two columns (10 bits: one) run in kernels
-    compiled for them, in tiles of another width in the general one: every kind,
-    with tables and on the fly, from two vectors, against the oracle."""
+    """Digits of 5 to 10 bits in tiles of two columns (10 bits, and variant 5 up to
+    9: one) run in kernels compiled for them, in tiles of another width in the
+    general one: every kind, with tables and on the fly, from two vectors, against
+    the oracle."""
     L = sum(digits)
-    compiled = [1 if k == 10 else 2 for k in digits]
-    general = [2 if k == 10 else 4 if k < 9 else 1 for k in digits]
+    compiled = [1 if k == 10 or variant == 5 else 2 for k in digits]
+    general = [2 if k == 10 or variant == 5 else 4 if k < 9 else 1 for k in digits]
     inputs = [rand_dev(F, L, 3000 + L), _edge_dev(F, L)]
     for kind in KINDS:
         want = [_oracle(F, X, kind) for X, _ in inputs]
