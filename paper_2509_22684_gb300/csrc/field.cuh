@@ -350,12 +350,12 @@ __device__ __forceinline__ void row_product(uint32_t E[8], uint32_t O[8], uint32
 //                            wide multiply fewer (80.3 against 79.4 G/s).
 //   r_0 = 2^32 - 2^28 + 1 (r' = 2^32 - 2^28 - 1): m and the high word
 //                            m - (m >> 4) of m r_0 come from shifts and adds.
+//   any other r_0:           m = E_0 r' and both words of m r_0 by multiplies.
 // m = -E_0 is written as sub.cc: as a plain negation the assembler folds it
 // into the multiplies' operands, which splits every wide multiply-add in two
 // (232 instead of 182 instructions a product).
 template <class F>
 __device__ __forceinline__ void row_reduce(uint32_t E[8], uint32_t O[8]) {
-    static_assert(F::P0 == 1u || F::P0 == 0xf0000001u, "no reduction row for this modulus");
     if constexpr (F::P0 == 1u && F::P1 == 0xffffffffu) {
         uint32_t m, h, z;
         asm("sub.cc.u32 %0, 0, %2;\n\t"
@@ -408,10 +408,13 @@ __device__ __forceinline__ void row_reduce(uint32_t E[8], uint32_t O[8]) {
             : "r"(E[0]), "r"(m), "n"(F::P1), "n"(F::P3), "n"(F::P5), "n"(F::P7), "n"(F::P2),
               "n"(F::P4), "n"(F::P6));
     } else {
-        const uint32_t m = 0u - E[0] - (E[0] << 28);
-        const uint32_t h = m - (m >> 4);  // high word of m r_0, without the carry of its low word
+        constexpr bool SHIFTS = F::P0 == 0xf0000001u;
+        const uint32_t m = SHIFTS ? 0u - E[0] - (E[0] << 28) : E[0] * F::RP;
+        // high word of m r_0, by shifts without the carry of its low word
+        const uint32_t h = SHIFTS ? m - (m >> 4) : __umulhi(m, F::P0);
+        const uint32_t l = SHIFTS ? m : m * F::P0;
         uint32_t z;
-        asm("add.cc.u32     %14, %16, %17;\n\t"
+        asm("add.cc.u32     %14, %16, %26;\n\t"
             "addc.cc.u32    %15, %15, %18;\n\t"
             "madc.lo.cc.u32  %8, %17, %23, %8;\n\t"
             "madc.hi.cc.u32  %9, %17, %23, %9;\n\t"
@@ -432,7 +435,7 @@ __device__ __forceinline__ void row_reduce(uint32_t E[8], uint32_t O[8]) {
               "+r"(O[7]), "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]),
               "=&r"(z), "+r"(E[1])
             : "r"(E[0]), "r"(m), "r"(h), "n"(F::P1), "n"(F::P3), "n"(F::P5), "n"(F::P7),
-              "n"(F::P2), "n"(F::P4), "n"(F::P6));
+              "n"(F::P2), "n"(F::P4), "n"(F::P6), "r"(l));
     }
 }
 
@@ -613,6 +616,22 @@ __device__ __forceinline__ void mul_high(uint32_t q[8], const uint32_t x[8], con
           "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]));
 }
 
+// low 256 bits of x w
+__device__ __forceinline__ void mul_low(uint32_t t[8], const uint32_t x[8], const uint32_t w[8]) {
+    asm("{\n\t.reg .u32 e<16>, o<16>;\n\t.reg .u64 t;\n\t"
+        ZK_NAME8(x, "%8", "%9", "%10", "%11", "%12", "%13", "%14", "%15")
+        ZK_NAME8(w, "%16", "%17", "%18", "%19", "%20", "%21", "%22", "%23")
+        ZK_ROW_LOW_NEW ZK_ROWS_LOW
+        "mov.u32 %0, e0;\n\t"
+        "add.cc.u32 %1, e1, o1;\n\taddc.cc.u32 %2, e2, o2;\n\t"
+        "addc.cc.u32 %3, e3, o3;\n\taddc.cc.u32 %4, e4, o4;\n\t"
+        "addc.cc.u32 %5, e5, o5;\n\taddc.cc.u32 %6, e6, o6;\n\taddc.u32 %7, e7, o7;\n\t}"
+        : "=&r"(t[0]), "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]),
+          "=&r"(t[6]), "=&r"(t[7])
+        : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7]),
+          "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]));
+}
+
 // t = x w + q (2^256 - r) mod 2^256
 template <class F>
 __device__ __forceinline__ void mul_low_fold(uint32_t t[8], const uint32_t x[8], const uint32_t w[8],
@@ -655,9 +674,21 @@ __device__ __forceinline__ void mul_low_fold(uint32_t t[8], const uint32_t x[8],
     } else if constexpr (F::P0 == 1u) {
         asm(ZK_LOW_HEAD ZK_LOW_Q ZK_ROW_LOW_ADD ZK_ROWS_LOW ZK_ROWS_N1 ZK_LOW_TAIL
             ZK_LOW_OPERANDS(0, ~F::P1));
-    } else {
+    } else if constexpr (F::P0 == 0xf0000001u) {
         asm(ZK_LOW_HEAD ZK_LOW_Q28 ZK_ROW_LOW_ADD ZK_ROWS_LOW ZK_ROWS_N1 ZK_LOW_TAIL
             ZK_LOW_OPERANDS(0, ~F::P1));
+    } else {  // any other lowest limb
+        const uint32_t n[8] = {0u - F::P0, ~F::P1, ~F::P2, ~F::P3, ~F::P4, ~F::P5, ~F::P6, ~F::P7};
+        uint32_t a[8], b[8];
+        mul_low(a, x, w);
+        mul_low(b, q, n);
+        uint64_t c = 0;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            c += uint64_t(a[i]) + b[i];
+            t[i] = uint32_t(c);
+            c >>= 32;
+        }
     }
 #undef ZK_LOW_HEAD
 #undef ZK_LOW_Q
@@ -680,22 +711,6 @@ __device__ __forceinline__ void mul_factor(uint32_t r[8], const uint32_t x[8], c
     mul_low_fold<F>(t, x, f.w, q);
 #pragma unroll
     for (int i = 0; i < 8; i++) r[i] = t[i];
-}
-
-// low 256 bits of x w
-__device__ __forceinline__ void mul_low(uint32_t t[8], const uint32_t x[8], const uint32_t w[8]) {
-    asm("{\n\t.reg .u32 e<16>, o<16>;\n\t.reg .u64 t;\n\t"
-        ZK_NAME8(x, "%8", "%9", "%10", "%11", "%12", "%13", "%14", "%15")
-        ZK_NAME8(w, "%16", "%17", "%18", "%19", "%20", "%21", "%22", "%23")
-        ZK_ROW_LOW_NEW ZK_ROWS_LOW
-        "mov.u32 %0, e0;\n\t"
-        "add.cc.u32 %1, e1, o1;\n\taddc.cc.u32 %2, e2, o2;\n\t"
-        "addc.cc.u32 %3, e3, o3;\n\taddc.cc.u32 %4, e4, o4;\n\t"
-        "addc.cc.u32 %5, e5, o5;\n\taddc.cc.u32 %6, e6, o6;\n\taddc.u32 %7, e7, o7;\n\t}"
-        : "=&r"(t[0]), "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]),
-          "=&r"(t[6]), "=&r"(t[7])
-        : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7]),
-          "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]));
 }
 
 // The factor of a constant given in Montgomery form, m = w R mod r, R = 2^256:
