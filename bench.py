@@ -19,6 +19,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -54,16 +55,27 @@ def measured_peaks() -> dict:
         return {}
 
 
-# the sources the timed pass kernel is compiled from (BLS12-381 instantiation)
+# the sources the timed pass kernel is compiled from (BLS12-381 instantiation);
+# what they include of their own folder counts too (kernel_source_hash)
 PASS_KERNEL_SOURCES = ("field.cuh", "ntt_pass.cuh", "kernels_bls12_381.cu")
 
 
 def kernel_source_hash() -> str:
-    h = hashlib.sha256()
+    """Key of a recorded capture: the pass kernel's sources and every header of
+    their folder that they include, directly or not (the block size and register
+    budget a kernel is compiled for stand in one of those)."""
     csrc = os.path.join(ROOT, "paper_2509_22684_gb300", "csrc")
-    for name in PASS_KERNEL_SOURCES:
+    todo, seen = list(PASS_KERNEL_SOURCES), {}
+    while todo:
+        name = todo.pop()
+        if name in seen:
+            continue
         with open(os.path.join(csrc, name), "rb") as f:
-            h.update(name.encode() + f.read())
+            seen[name] = f.read()
+        todo += re.findall(r'^\s*#\s*include\s+"([^"]+)"', seen[name].decode(), re.M)
+    h = hashlib.sha256()
+    for name in sorted(seen):
+        h.update(name.encode() + seen[name])
     return h.hexdigest()[:16]
 
 

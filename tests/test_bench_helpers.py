@@ -3,7 +3,10 @@ for the same pass-kernel sources and schedule, the tuned-schedule lookup reads
 the shipped table, clock samples are kept only inside the timed region."""
 import json
 import os
+import shutil
 import sys
+
+import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 if ROOT not in sys.path:
@@ -44,6 +47,20 @@ def test_kernel_source_hash_covers_the_pass_kernel_sources():
     h = bench.kernel_source_hash()
     assert len(h) == 16 and int(h, 16) >= 0
     assert bench.kernel_source_hash() == h      # deterministic
+
+
+@pytest.mark.parametrize("name", ["field.cuh", "ntt_pass.cuh", "field_kernels.cuh", "kernels.h"])
+def test_kernel_source_hash_changes_with_every_file_of_the_kernel(tmp_path, monkeypatch, name):
+    """The block size and register budget of the timed kernel stand in a header
+    that its translation unit includes: a change there makes the record stale."""
+    h = bench.kernel_source_hash()
+    csrc = os.path.join("paper_2509_22684_gb300", "csrc")
+    shutil.copytree(os.path.join(ROOT, csrc), tmp_path / csrc)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert bench.kernel_source_hash() == h
+    with open(tmp_path / csrc / name, "a") as f:
+        f.write("// changed\n")
+    assert bench.kernel_source_hash() != h
 
 
 def test_clock_sampler_keeps_only_samples_inside_the_timed_region(tmp_path):
