@@ -96,12 +96,12 @@ typedef struct {
  *                Montgomery-form limbs (host memory, read during the call);
  *                must be nonzero and canonical.
  * The plan owns its device twiddle tables (allocated and filled here, freed by
- * zkntt_plan_destroy).  Without a tuned schedule or an explicit mode, the
- * inter-pass twiddles are precomputed tables (n entries for the first pass)
- * when those fit beside three vectors in the device memory free at creation,
- * else formed on the fly from split-exponent tables of about 2 sqrt(n)
- * entries.  Returns EINVAL on bad arguments, ENOMEM when the tables do not
- * fit, ECUDA on other CUDA failures.
+ * zkntt_plan_destroy).  Without an explicit mode the inter-pass twiddles are
+ * precomputed tables (64 bytes an entry, n entries for the first pass) when
+ * those fit beside three vectors in the device memory free at creation, else
+ * formed on the fly from split-exponent tables of about 2 sqrt(n) entries
+ * (also where a tuned schedule names precomputed ones).  Returns EINVAL on bad
+ * arguments, ENOMEM when the tables do not fit, ECUDA on other CUDA failures.
  */
 zkntt_status zkntt_plan_create(zkntt_plan *out, zkntt_field field, int log_n, zkntt_dir dir,
                                const uint32_t *coset_shift);

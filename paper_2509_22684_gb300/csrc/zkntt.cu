@@ -619,11 +619,13 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
     }
     const int p = P->passes;
     if (!ilp) ilp = default_ilp(L, p);
-    if (mode == ZKNTT_TWIDDLE_AUTO && p > 1) {
-        // Precomputed inter-pass tables (pass i: 2^(K_i + lo_bits_i) entries of
-        // 64 bytes; pass 1's is n entries) unless they would not fit beside the input,
-        // output and scratch vectors in the device memory free now: then the
-        // split-exponent tables (about 2 sqrt(n_i) entries) instead.
+    const bool mode_open = !(opts && opts->twiddle_mode);
+    if (mode_open && mode != ZKNTT_TWIDDLE_OTF && p > 1) {
+        // The caller leaves the mode open: precomputed inter-pass tables (pass i:
+        // 2^(K_i + lo_bits_i) entries of 64 bytes; pass 1's is n entries) unless they
+        // would not fit beside the input, output and scratch vectors in the device
+        // memory free now: then the split-exponent tables (about 2 sqrt(n_i) entries)
+        // instead, whatever mode a tuned schedule names.
         size_t fr = 0, tot = 0;
         ZK_CHECK(cudaMemGetInfo(&fr, &tot));
         size_t tables = 0;

@@ -307,6 +307,53 @@ def test_execute_host_buffered_matches_device_execution(F):
             p.execute_host_buffered(xh, yh, work[:8 * (1 << L)], stream=s)
 
 
+def test_auto_twiddles_when_device_memory_is_short():
+    """With half a gigabyte of device memory free beside the vectors: the 64-byte
+    factors of the tuned schedule's tables at 2^24 (1.1 GB) do not fit, so a plan
+    whose mode is left open forms them on the fly and runs, as do the Groth16
+    sequence's own plans at 2^22; a plan that asks for the tables is refused."""
+    import torch
+    import paper_2509_22684_gb300 as zk
+    from paper_2509_22684_gb300 import ZkNttError
+    F, L = fld.BLS12_381, 24
+    x = rand_dev(F, L, 2424)[1]
+    y = torch.empty_like(x)
+    with _plan(F, L, "ntt") as p:
+        assert p.describe()["twiddle_mode"] == "precomp"
+        want = p.execute(x)
+    G, M = fld.BLS12_377, 22
+    abc = [rand_dev(G, M, 2200 + k)[1] for k in range(3)]
+    h = torch.empty_like(abc[0])
+    scratch = torch.empty((3 << M, 8), dtype=torch.int32, device="cuda")
+    with _plan(G, M, "intt") as i, _plan(G, M, "coset_ntt") as c, _plan(G, M, "coset_intt") as ci:
+        A, B, C = (c.execute(i.execute(v)) for v in abc)
+        z = G.to_mont(pow(pow(G.g, 1 << M, G.r) - 1, -1, G.r))
+        want_h = ci.execute(zk.pointwise(G.name, A, B, C, z))
+        torch.cuda.synchronize()
+        del A, B, C
+    fill = []
+    try:
+        for _ in range(4):      # (the allocator rounds sizes)
+            torch.cuda.empty_cache()
+            more = torch.cuda.mem_get_info()[0] - 500 * 1000 * 1000
+            if more < 64 << 20:
+                break
+            fill.append(torch.empty(more, dtype=torch.uint8, device="cuda"))
+        with _plan(F, L, "ntt") as p:
+            assert p.describe()["twiddle_mode"] == "otf"
+            p.execute(x, y)
+            torch.cuda.synchronize()
+        with pytest.raises(ZkNttError):
+            zk.Plan(F.name, L, twiddle_mode="precomp")
+        zk.groth16_h(G.name, M, *abc, h=h, scratch=scratch)
+        torch.cuda.synchronize()
+    finally:
+        fill.clear()
+        torch.cuda.empty_cache()
+    assert torch.equal(y, want)
+    assert torch.equal(h, want_h)
+
+
 def test_bls12_381_2_30_beyond_the_tuned_sizes():
     """2^30 BLS12-381 F_r (32 GiB per vector; sizes above 2^28 run with the
     planner's default split and pick their twiddle mode by free memory):
