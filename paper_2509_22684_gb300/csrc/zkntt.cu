@@ -313,18 +313,6 @@ zkntt_status device_info(DeviceInfo **out) {
     DeviceInfo &d = g_devices[dev];
     if (!d.init) {
         ZK_CHECK(cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev));
-        for (int f = 0; f < NUM_FIELDS; f++)
-            for (const void *k : {field_kernels(f).any4, field_kernels(f).any2})
-                ZK_CHECK(cudaFuncSetAttribute(k,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              PASS_MAX_SMEM));
-        for (int f = 0; f < NUM_FIELDS; f++)
-            for (const auto &table : {field_kernels(f).fixed, field_kernels(f).wide})
-                for (int d = 0; d <= MAX_DIGIT_BITS; d++)
-                    for (const void *k : table[d])
-                        if (k)
-                            ZK_CHECK(cudaFuncSetAttribute(
-                                k, cudaFuncAttributeMaxDynamicSharedMemorySize, PASS_MAX_SMEM));
         for (int f = 0; f < NUM_FIELDS; f++) {
             ZK_CHECK(cudaFuncSetAttribute(batch_kernel_ptr(f),
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -554,6 +542,11 @@ zkntt_status set_launch(const PassPlan *ps, PassLaunch *r, int field, Kind kind,
         r->kernel = ps->ilp == 5 ? kk.any2 : kk.any4;
         r->threads = int(pass_threads_for(uint32_t(ps->K), uint32_t(ps->log_cols), ps->ilp));
     }
+    // Set per plan, not for all kernels at device set-up: that loads every kernel of
+    // every field, 32 ms of a process's first plan (35 -> 3.5 ms with the device code
+    // uncompressed in the library; the kernels of one field take 1.8).
+    ZK_CHECK(cudaFuncSetAttribute(r->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  PASS_MAX_SMEM));
     // the twiddle table and the tile buffers
     const size_t tile_bytes = size_t(16) * tile_units(1u << (ps->K + ps->log_cols));
     const size_t table_bytes = size_t(64) * tab_entries(uint32_t(ps->K));
