@@ -619,15 +619,16 @@ zkntt_status build_plan(zkntt_plan_s *P, const zkntt_plan_options *opts) {
         // would not fit beside the input, output and scratch vectors in the device
         // memory free now: then the split-exponent tables (about 2 sqrt(n_i) entries)
         // instead, whatever mode a tuned schedule names.
-        size_t fr = 0, tot = 0;
-        ZK_CHECK(cudaMemGetInfo(&fr, &tot));
-        size_t tables = 0;
+        size_t need = 3 * (size_t(32) << L);
         for (int i = 0, hb = 0; i < p - 1; i++) {
             hb += k[i];
-            tables += size_t(64) << (L - hb + k[i]);
+            need += size_t(64) << (L - hb + k[i]);
         }
-        const size_t vectors = 3 * (size_t(32) << L);
-        if (tables + vectors > fr) mode = ZKNTT_TWIDDLE_OTF;
+        // (not asked below 32 MiB, up to 2^17: the query takes 5 to 10 us, and such a
+        // plan 75 to 250)
+        size_t fr = need, tot = 0;
+        if (need >= size_t(32) << 20) ZK_CHECK(cudaMemGetInfo(&fr, &tot));
+        if (need > fr) mode = ZKNTT_TWIDDLE_OTF;
     }
     if (mode != ZKNTT_TWIDDLE_OTF) mode = ZKNTT_TWIDDLE_PRECOMP;
     P->mode = mode;
