@@ -41,7 +41,6 @@ constexpr uint32_t BATCH_STATUS_TIMEOUT = 4u;  // == ZKNTT_ETIMEOUT
 
 struct BatchSeg {
     PassArgs a;
-    uint32_t K;           // digit bits of this pass
     uint32_t first_item;  // index of the segment's first tile in the work list
     int32_t dep;          // segment that must be complete first (-1: none)
     uint32_t dep_tiles;   // its tiles

@@ -725,12 +725,6 @@ __device__ __forceinline__ void make_factor(Factor &f, const uint32_t m[8], cons
 
 // ---------------------------------------------------------------------------
 // element load/store: 32 bytes as two 16-byte vectors
-__device__ __forceinline__ void ld_elem(uint32_t x[8], const uint4 *p) {
-    uint4 lo = p[0], hi = p[1];
-    x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w;
-    x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
-}
-
 __device__ __forceinline__ void ldg_elem(uint32_t x[8], const uint4 *p) {
     uint4 lo = __ldg(p), hi = __ldg(p + 1);
     x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w;

@@ -7,6 +7,8 @@
 
 namespace zkntt {
 
+static_assert(NUM_KINDS == PASS_KINDS, "the kernel tables have a place for every kind");
+
 // the pass kernels compiled for a digit of K bits: one thread per four elements
 // of a tile, 128 registers (2^24: 2594 us, with 96 2606, with 80 2702)
 template <class F, int K, Kind KIND>

@@ -6,12 +6,13 @@
 namespace zkntt {
 
 constexpr int MAX_DIGIT_BITS = 11;  // largest sub-transform a block holds (2^11 x 32 B = 64 KiB)
-constexpr int MAX_TILE_BITS = 11;   // tiles hold at most 2^11 elements (C x 2^K)
+constexpr int PASS_KINDS = 6;       // values of Kind (ntt_pass.cuh)
 
 struct FieldKernels {
     const void *any4, *any2;  // the pass kernels of runtime sizes: radix 4, radix 2 (variant 5)
-    const void *fixed[MAX_DIGIT_BITS + 1][6];  // pass kernels by digit bits and Kind (null: none)
-    const void *wide[MAX_DIGIT_BITS + 1][6];   // the same with one thread per pair (variant 5)
+    // pass kernels by digit bits and Kind (null: none), and those with one thread per pair (variant 5)
+    const void *fixed[MAX_DIGIT_BITS + 1][PASS_KINDS];
+    const void *wide[MAX_DIGIT_BITS + 1][PASS_KINDS];
     const void *gen_powers;
     const void *gen_twiddle;
     const void *field_op;

@@ -1003,7 +1003,6 @@ zkntt_status launch_batch_field(const std::vector<JobSpec> &jobs, cudaStream_t s
         sg.a = pass_args(P, i, src, dst);
         sg.a.log_cols = uint32_t(batch_log_cols(P, i));
         sg.a.num_tiles = batch_tiles(P, i);
-        sg.K = uint32_t(P->ps[i].K);
         sg.first_item = item;
         sg.ntiles = sg.a.num_tiles;
         sg.job = job_ids[segs[k].job];
@@ -1559,7 +1558,6 @@ zkntt_status zkntt_inject_timeout(int timeout_ms, void *stream) {
     tab->nseg = 1;
     tab->total_items = 1;
     tab->timeout_ns = (unsigned long long)timeout_ms * 1000000ull;
-    tab->seg[0].K = 4;
     tab->seg[0].first_item = 0;
     tab->seg[0].dep = 0;
     tab->seg[0].dep_tiles = 1;
