@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(128) block_dft_kernel(const uint4 *in, uint4 *
     }
 }
 
-// c = op(a, b) elementwise: 0 mul, 1 add, 2 sub
+// c = op(a, b) elementwise: 0 mul, 1 add, 2 sub, 3 sub_lazy
 template <class F>
 __global__ void field_op_kernel(int op, const uint4 *a, const uint4 *b, uint4 *c, size_t n) {
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;

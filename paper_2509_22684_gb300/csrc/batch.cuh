@@ -26,8 +26,9 @@ namespace zkntt {
 
 constexpr int BATCH_MAX_SEGMENTS = 160;
 constexpr uint32_t BATCH_THREADS = 256;
-// blocks per SM the register budget is compiled for (80 registers a thread: 64
-// uneven transforms of 2^10..2^20 in 1824 us; 64 registers 1926, 128 2042)
+// blocks per SM the register budget is compiled for (80 registers a thread, which
+// spill 112 to 208 bytes of stores: 64 uneven transforms of 2^10..2^20 in 1824 us;
+// 64 registers 1926, 128 and two blocks, with nothing to cover a tile's loads, 2042)
 #ifndef ZKNTT_BATCH_MIN_BLOCKS
 #define ZKNTT_BATCH_MIN_BLOCKS 3
 #endif

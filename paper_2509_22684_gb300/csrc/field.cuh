@@ -2,7 +2,9 @@
 //
 // Elements are 256-bit little-endian limb vectors in Montgomery form
 // (X = x * 2^256 mod r), as the paper describes field elements: word-sized
-// limbs (Section II), results of every field operation in [0, r).
+// limbs (Section II).  mul, add and sub give results in [0, r); the operations of a
+// transform (the _loose ones and mul_factor) keep residues in [0, 2r), or below 4r for
+// a difference that only feeds a product, and its last pass brings the outputs below r.
 //
 // * mul: Montgomery product X * Y * 2^-256 mod r, coarsely integrated operand
 //   scanning (CIOS): for each limb b_i, t += a * b_i, then m = t_0 * r' and
@@ -255,7 +257,7 @@ __device__ __forceinline__ void diff_loose(uint32_t r[8], const uint32_t a[8], c
 }
 
 // r = a + p - b, in (0, 2p) and congruent to a - b, for canonical a, b: no
-// conditional correction.  Only for values that feed mul as its second
+// conditional correction (the G-point block transforms).  Only for values that feed mul as its second
 // (limb-scanned) operand, which may be any value below 2^256.
 template <class F>
 __device__ __forceinline__ void sub_lazy(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {

@@ -23,8 +23,9 @@
 // element's output factor and the store to global memory.  Tiles with more than
 // one thread per four elements (small transforms, where warps in flight count)
 // take the stages one by one, one butterfly a thread.
-// The difference x - y is formed as x + r - y with no conditional correction:
-// it only feeds the product, which takes any x below 2r.
+// A difference that only feeds a product is formed as x + 2r - y, below 4r, without a
+// correction where 4r < 2^256 (BN254, BLS12-377), else corrected by 2r (BLS12-381): the
+// product takes any x up to 2^256 - 2^228.
 // Digits of 5 to 10 bits in the usual tile width have kernels compiled for them;
 // every other digit and width is served by kernels whose sizes are runtime values.
 //
